@@ -155,15 +155,19 @@ int lbs_set_initial(lbs_handle *h, const double *u0, const double *v0);
 int lbs_set_initial_device(lbs_handle *h, const double *u0, const double *v0);
 
 /* Advance n >= 0 iterations (asynchronous).  Launches one fused kernel per
- * iteration, replayed from a CUDA graph in chunks (lbs_set_graph_chunk).
+ * iteration, replayed from a CUDA graph in chunks (lbs_set_graph_chunk).  A
+ * small lattice (up to some 77 000 nodes in single precision, 19 000 in double)
+ * instead advances all n, up to the point where a monitor is due, in one
+ * cooperative launch, unless lbs_set_variant chose its kernel or the graph
+ * chunk is 0; the results are the same bits.
  * Returns LBS_EUNSTABLE if an earlier monitor already found a non-finite
  * value; the state then stays available for lbs_fields. */
 int lbs_step(lbs_handle *h, int64_t n);
 
 /* Wait for the handle's work; LBS_EUNSTABLE if a monitor found a
  * non-finite value (lbs_unstable_iteration tells where), LBS_ETIMEOUT if a
- * kernel gave up waiting for its tile copies (bounded wait; the state is then
- * not advanced for the affected tiles). */
+ * kernel gave up waiting for its tile copies or for its other blocks (bounded
+ * wait; the state is then not advanced for the affected tiles). */
 int lbs_sync(lbs_handle *h);
 
 /* Fields at the current iteration into caller-owned HOST buffers (any may be
@@ -236,8 +240,8 @@ int lbs_grid_error_device(lbs_handle *h, const double *u_ref, double out[2]);
  * LBS_EUNSTABLE. */
 int lbs_set_monitor_interval(lbs_handle *h, int64_t m);
 
-/* Iterations per captured CUDA graph (even, >= 2; 0 launches directly).
- * Default 64. */
+/* Iterations per captured CUDA graph (even, >= 2; 0 launches every iteration
+ * directly).  Default 64. */
 int lbs_set_graph_chunk(lbs_handle *h, int32_t k);
 
 /* Kernel tile variant (an index from lbs_tile_variants).  Each precision has a

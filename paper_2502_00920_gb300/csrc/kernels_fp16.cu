@@ -1,6 +1,7 @@
 // FP16 storage (scaled), FP32 arithmetic, u as a float pair: kernel instantiations and launchers of liblbs.
 #include "lbs_device.cuh"
 #include "lbs_batch.cuh"
+#include "lbs_resident.cuh"
 
 namespace lbs {
 namespace {
@@ -75,6 +76,18 @@ bool tma_maps(const Params &p, int v, const void *g, const void *u, void *og, vo
   return make_tma_maps<V4>(p, g, u, og, ou);
 }
 
+// resident launches: the tiles and lines of single precision (us per iteration
+// on walled neo-Hooke lattices, one lattice alone / three side by side, against
+// launching every iteration from a graph: 40 x 40 10.1 / 3.5 -> 2.8 / 0.94,
+// 128 x 128 10.5 / 3.7 -> 2.8 / 1.6, 256 x 256 10.8 / 4.8 -> 3.9 / 3.9)
+using RS = ResCfg<P, 16, 8>;
+using RL = ResCfg<P, 32, 16>;
+int resident_large(const Params &p) { return p.extrap ? resident_sms() / 2 : resident_sms(); }
+bool resident_applies(const Params &p) { return resident_shape<RS, RL>(p, resident_large(p)) != kResidentNone; }
+cudaError_t resident(const Params &p, const ResidentPtrs &s, int parity, int64_t k0, int n, cudaStream_t st) {
+  return launch_resident<RS, RL>(p, s, parity, k0, n, resident_large(p), st);
+}
+
 // the server's batch tile shapes: the global-memory tiles V0-V3
 constexpr int kBatchShapes = 4;
 TileShape batch_shape(int b) { return shape(b); }
@@ -99,6 +112,8 @@ const Launchers kL = {kVariants,
                       iterations_per_call,
                       launch_step<V0>,
                       step_kernel_count<V0>,
+                      resident_applies,
+                      resident,
                       tma_maps,
                       launch_init<V0>,
                       launch_fields<V0>,

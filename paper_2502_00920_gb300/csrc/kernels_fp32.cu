@@ -1,6 +1,7 @@
 // FP32 storage and arithmetic, u as a float pair: kernel instantiations and launchers of liblbs.
 #include "lbs_device.cuh"
 #include "lbs_batch.cuh"
+#include "lbs_resident.cuh"
 
 namespace lbs {
 namespace {
@@ -94,6 +95,22 @@ bool tma_maps(const Params &p, int v, const void *g, const void *u, void *og, vo
   return make_tma_maps<V4>(p, g, u, og, ou);
 }
 
+// resident launches (us per iteration on walled neo-Hooke lattices, one lattice
+// alone / three advancing side by side; launching every iteration from a graph
+// before them): 32 x 32 9.1 / 3.1 -> 2.9 / 0.95 and 128 x 128 9.5 / 3.3 ->
+// 2.9 / 1.6 on 16 x 8 tiles, 160 x 160 10.7 / 4.2 -> 4.0 / 1.4 and 256 x 256
+// 9.5 / 4.2 -> 3.9 / 3.8 on 32 x 16 tiles (80 registers, one block per SM).
+// Two-point wall extrapolation: 160 x 40 11.8 / 4.5 -> 4.7 / 1.6; its large
+// tiles lose beside others once they fill the GPU (391 x 173 12.3 / 5.4 -> 7.2
+// / 7.1), so they stop at half.
+using RS = ResCfg<P, 16, 8>;
+using RL = ResCfg<P, 32, 16>;
+int resident_large(const Params &p) { return p.extrap ? resident_sms() / 2 : resident_sms(); }
+bool resident_applies(const Params &p) { return resident_shape<RS, RL>(p, resident_large(p)) != kResidentNone; }
+cudaError_t resident(const Params &p, const ResidentPtrs &s, int parity, int64_t k0, int n, cudaStream_t st) {
+  return launch_resident<RS, RL>(p, s, parity, k0, n, resident_large(p), st);
+}
+
 // the server's batch tile shapes: the global-memory tiles V0-V3
 constexpr int kBatchShapes = 4;
 TileShape batch_shape(int b) { return shape(b); }
@@ -118,6 +135,8 @@ const Launchers kL = {kVariants,
                       iterations_per_call,
                       launch_step<V0>,
                       step_kernel_count<V0>,
+                      resident_applies,
+                      resident,
                       tma_maps,
                       launch_init<V0>,
                       launch_fields<V0>,

@@ -1,6 +1,7 @@
 // FP64 storage and arithmetic: kernel instantiations and launchers of liblbs.
 #include "lbs_device.cuh"
 #include "lbs_batch.cuh"
+#include "lbs_resident.cuh"
 
 namespace lbs {
 namespace {
@@ -57,6 +58,22 @@ bool tma_maps(const Params &p, int v, const void *g, const void *u, void *og, vo
   return make_tma_maps<V4>(p, g, u, og, ou);
 }
 
+// resident launches (us per iteration on walled neo-Hooke lattices, one lattice
+// alone / three side by side, against launching every iteration from a graph):
+// 40 x 40 26.4 / 8.9 -> 9.2 / 3.1, 160 x 40 26.2 / 8.8 -> 9.0 / 4.2 and 96 x 96
+// 31.6 / 11.1 -> 9.1 / 6.6 on 8 x 8 tiles, 128 x 128 31.6 / 11.4 -> 19.7 / 9.9 on
+// 16 x 16 tiles.  FP64 operations bound both (a warp's operation holds its
+// scheduler's FP64 unit for tens of cycles), so a tile's halo is dear: past
+// half the SMs the 16 x 16 tiles lose beside others (160 x 160 31.6 / 15.1 ->
+// 19.7 / 19.6), and with the two-point wall extrapolation they do not pay.
+using RS = ResCfg<P, 8, 8>;
+using RL = ResCfg<P, 16, 16>;
+int resident_large(const Params &p) { return p.extrap ? 0 : resident_sms() / 2; }
+bool resident_applies(const Params &p) { return resident_shape<RS, RL>(p, resident_large(p)) != kResidentNone; }
+cudaError_t resident(const Params &p, const ResidentPtrs &s, int parity, int64_t k0, int n, cudaStream_t st) {
+  return launch_resident<RS, RL>(p, s, parity, k0, n, resident_large(p), st);
+}
+
 // the server's batch tile shapes: the global-memory tiles V0-V3
 constexpr int kBatchShapes = 4;
 TileShape batch_shape(int b) { return shape(b); }
@@ -81,6 +98,8 @@ const Launchers kL = {kVariants,
                       iterations_per_call,
                       launch_step<V0>,
                       step_kernel_count<V0>,
+                      resident_applies,
+                      resident,
                       tma_maps,
                       launch_init<V0>,
                       launch_fields<V0>,

@@ -238,6 +238,9 @@ using namespace lbs;
 
 namespace {
 
+// iterations of one resident launch at most (a few tens of milliseconds)
+constexpr int kResidentMost = 4096;
+
 StepPtrs ptrs(const lbs_handle *h, int parity, const int64_t *kptr, int64_t koff) {
   StepPtrs s;
   s.g_in = h->g[parity];
@@ -502,7 +505,11 @@ int lbs_create(const lbs_lattice *lat, const lbs_material *mat, const lbs_bcs *b
   h->errdev = (int *)(h->kdev + 2);
   h->bytes = 2 * (s.g + s.u + s.b) + s.mon;
   rc = select_variant(h, h->L->default_variant);
-  if (!rc && cudaMemsetAsync(h->zero_dev, 0, 2 * sizeof(int64_t), h->stream) != cudaSuccess) rc = LBS_ECUDA;
+  // mon_out[7] holds the resident launches' barrier counters
+  if (!rc && (cudaMemsetAsync(h->zero_dev, 0, 2 * sizeof(int64_t), h->stream) != cudaSuccess ||
+              cudaMemsetAsync(h->mon_out + 7, 0, sizeof(double), h->stream) != cudaSuccess))
+    rc = LBS_ECUDA;
+  h->resident = h->L->resident_applies(h->P);
   if (!rc) rc = lbs_set_initial_device(h, nullptr, nullptr);
   if (!rc && cudaStreamSynchronize(h->stream) != cudaSuccess) rc = fail(LBS_ECUDA, "initialisation failed");
   if (rc) {
@@ -593,7 +600,28 @@ int lbs_step(lbs_handle *h, int64_t n) {
   int rc = check_monitor(h, false);
   if (rc) return rc;
   while (n > 0) {
-    if (h->graph_chunk > 0 && n >= h->graph_chunk) {
+    if (h->resident && h->graph_chunk > 0) {
+      // the iterations up to the end or the point where a monitor is due: the
+      // first boundary at or after it of the graph chunks (and of the single
+      // iterations that follow them)
+      int m = 0;
+      do {
+        m += n - m >= h->graph_chunk ? h->graph_chunk : 1;
+      } while (m < n && m < kResidentMost && !(h->mon_interval > 0 && h->k + m >= h->next_mon));
+      ResidentPtrs rp;
+      for (int i = 0; i < 2; ++i) {
+        rp.g[i] = h->g[i];
+        rp.u[i] = h->u[i];
+        rp.b[i] = h->b[i];
+      }
+      rp.bar = (unsigned *)(h->mon_out + 7);
+      rp.err = h->errdev;
+      LBS_CK(h->L->resident(h->P, rp, h->parity, h->k, m, h->stream));
+      h->launches += 1;
+      h->parity ^= m & 1;
+      h->k += m;
+      n -= m;
+    } else if (h->graph_chunk > 0 && n >= h->graph_chunk) {
       if (!h->graph[h->parity] || h->graph_variant[h->parity] != h->variant) {
         if (h->graph[h->parity]) {
           cudaGraphExecDestroy(h->graph[h->parity]);
@@ -787,7 +815,9 @@ int lbs_set_graph_chunk(lbs_handle *h, int32_t k) {
 int lbs_set_variant(lbs_handle *h, int32_t variant) {
   if (!h || variant < 0 || variant >= h->L->nvariants) return fail(LBS_EINVAL, "unknown tile variant");
   if (variant != h->variant) LBS_CK(cudaStreamSynchronize(h->stream));
-  return select_variant(h, variant);
+  const int rc = select_variant(h, variant);
+  if (!rc) h->resident = false;  // the caller's choice of step kernel
+  return rc;
 }
 
 int lbs_autotune_handle(lbs_handle *h, int32_t steps) {
@@ -795,7 +825,11 @@ int lbs_autotune_handle(lbs_handle *h, int32_t steps) {
   int32_t best = 0;
   int rc = lbs_autotune(&h->lat, &h->mat, &h->bcs, steps, &best, nullptr);
   if (rc) return rc;
-  return lbs_set_variant(h, best);
+  rc = lbs_set_variant(h, best);
+  // the variants are what single launches run on; a small lattice's longer
+  // runs stay resident
+  if (!rc) h->resident = h->L->resident_applies(h->P);
+  return rc;
 }
 
 // ---- checkpoint / resume

@@ -60,6 +60,43 @@ __device__ __forceinline__ float gload(const float *p, size_t i, float) { return
 // FP16 storage: the kernels work in units of g * 2^gshift (exact power-of-two
 // scaling), so loads and stores only convert
 __device__ __forceinline__ float gload(const __half *p, size_t i, float) { return __half2float(__ldg(p + i)); }
+// The same loads in a kernel that also writes the arrays it reads (the resident
+// kernel: iteration k + 1 reads what other blocks stored in iteration k of the
+// same launch), where the read-only path above would be wrong: ordinary
+// loads, ordered by the grid barrier's acquire.  COH picks them.
+__device__ __forceinline__ double ld_coh(const double *p) {
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float ld_coh(const float *p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ __half ld_coh(const __half *p) {
+  unsigned short v;
+  asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
+  return __ushort_as_half(v);
+}
+__device__ __forceinline__ double2 ld_coh(const double2 *p) {
+  double2 v;
+  asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float4 ld_coh(const float4 *p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double half_wide(double v) { return v; }
+__device__ __forceinline__ float half_wide(float v) { return v; }
+__device__ __forceinline__ float half_wide(__half v) { return __half2float(v); }
+template <bool COH, class G, class R>
+__device__ __forceinline__ R gld(const G *p, size_t i, R inv) {
+  if constexpr (COH) return half_wide(ld_coh(p + i));
+  else return gload(p, i, inv);
+}
 __device__ __forceinline__ void gstore(double *p, size_t i, double v, double) { p[i] = v; }
 __device__ __forceinline__ void gstore(float *p, size_t i, float v, float) { p[i] = v; }
 __device__ __forceinline__ void gstore(__half *p, size_t i, float v, float) { p[i] = __float2half_rn(v); }
@@ -264,11 +301,30 @@ __device__ inline void edge_value(const Params &P, int e, int64_t k, double out[
 // carried to the wall(s) the link crosses as v + (v - v_in)/2 per crossed
 // wall, v_in the value at the next node inwards along that wall's normal: r
 // and Pi from that node's own g, N from the side array's second layer.
-template <class R, class G, bool LIN>
-__device__ void wall_rules(const Params &P, const R *bnd, const G *g, const double (*sev)[2], int x, int y,
-                           const R g0[9], unsigned mask, R f[9], R gsc) {
-  int xw, yw;
-  walls_of(P, x, y, xw, yw);
+// wn: N11, N21 of the x wall's side entry and N22, N12 of the y wall's (wall_n,
+// loaded by the caller; only those of a Neumann wall the node sits on are used).
+template <bool COH, class R>
+__device__ __forceinline__ void wall_n(const Params &P, const R *bnd, int xw, int yw, int x, int y, R wn[4]) {
+  auto ld = [&](size_t i) -> R {
+    if constexpr (COH) return ld_coh(bnd + i);
+    else return bnd[i];
+  };
+  wn[0] = wn[1] = wn[2] = wn[3] = R(0);
+  if (xw >= 0 && P.etype[xw] == LBS_NEUMANN) {
+    const size_t o = side_entry(P, 0, xw, y);
+    wn[0] = ld(o);
+    wn[1] = ld(o + 2);
+  }
+  if (yw >= 0 && P.etype[yw] == LBS_NEUMANN) {
+    const size_t o = side_entry(P, 0, yw, x);
+    wn[2] = ld(o + 3);
+    wn[3] = ld(o + 1);
+  }
+}
+
+template <class R, class G, bool LIN, bool COH>
+__device__ void wall_rules(const Params &P, const R *bnd, const G *g, const double (*sev)[2], int x, int y, int xw,
+                           int yw, const R wn[4], const R g0[9], unsigned mask, R f[9], R gsc) {
   const bool xn = xw >= 0 && P.etype[xw] == LBS_NEUMANN;
   const bool yn = yw >= 0 && P.etype[yw] == LBS_NEUMANN;
   // Pi*/cs^2 from N and T* is brought into the units of g (times gsc)
@@ -287,18 +343,16 @@ __device__ void wall_rules(const Params &P, const R *bnd, const G *g, const doub
   const R Axx_o = R(3) * mxx, Axy_o = R(3) * mxy, Ayy_o = R(3) * myy;
   R Axx_x = 0, axy_x = 0, Ayy_y = 0, axy_y = 0;
   if (xn) {
-    const R *Nn = bnd + side_entry(P, 0, xw, y);  // N11, N12, N21, N22
     const double *T = sev[xw];
     const R s = (xw == kRight) ? R(1) : R(-1);
-    Axx_x = (Nn[0] - s * (R)T[0]) * ics2;
-    axy_x = (Nn[2] - s * (R)T[1]) * ics2;
+    Axx_x = (wn[0] - s * (R)T[0]) * ics2;
+    axy_x = (wn[1] - s * (R)T[1]) * ics2;
   }
   if (yn) {
-    const R *Nn = bnd + side_entry(P, 0, yw, x);
     const double *T = sev[yw];
     const R s = (yw == kTop) ? R(1) : R(-1);
-    Ayy_y = (Nn[3] - s * (R)T[1]) * ics2;
-    axy_y = (Nn[1] - s * (R)T[0]) * ics2;
+    Ayy_y = (wn[2] - s * (R)T[1]) * ics2;
+    axy_y = (wn[3] - s * (R)T[0]) * ics2;
   }
   // two-point extrapolation: half the differences own - inner of r, A and N
   // for the x wall (dX, nX) and the y wall (dY, nY) the node sits on (a
@@ -317,7 +371,7 @@ __device__ void wall_rules(const Params &P, const R *bnd, const G *g, const doub
       R ri = 0, ixx = 0, ixy = 0, iyy = 0;
 #pragma unroll
       for (int q = 0; q < 9; ++q) {
-        const R v = gload(g, q * plane + idx, R(1));
+        const R v = gld<COH>(g, q * plane + idx, R(1));
         ri += v;
         ixx += R(ex(q) * ex(q)) * v;
         ixy += R(ex(q) * ey(q)) * v;
@@ -325,8 +379,18 @@ __device__ void wall_rules(const Params &P, const R *bnd, const G *g, const doub
       }
       const R in[4] = {ri, R(3) * ixx, R(3) * ixy, R(3) * iyy};
       const int pos = w == 0 ? y : x;
-      const R *N0 = bnd + side_entry(P, 0, e, pos);
-      const R *N1 = bnd + side_entry(P, 1, e, pos);
+      R N0[4], N1[4];
+      const size_t o0 = side_entry(P, 0, e, pos), o1 = side_entry(P, 1, e, pos);
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        if constexpr (COH) {
+          N0[m] = ld_coh(bnd + o0 + m);
+          N1[m] = ld_coh(bnd + o1 + m);
+        } else {
+          N0[m] = bnd[o0 + m];
+          N1[m] = bnd[o1 + m];
+        }
+      }
       R *d = w == 0 ? dX : dY;
       R *n = w == 0 ? nX : nY;
 #pragma unroll
@@ -505,8 +569,8 @@ struct TileCfg : TileGeom<TX_, TY_, NTY_> {
 // first moments sum_q e_q g_q (own node, post-collision at k) and
 // sum_q e_q f_q (streamed, at k + 1).  EDGE: wrap, walls and boundary rules;
 // LIN: the two-point wall extrapolation (lattices with P.extrap set).
-template <class Pr, bool EDGE, bool LIN>
-__device__ __forceinline__ void gather(const Params &P, const typename Pr::gs *__restrict__ g, const typename Pr::real *bnd,
+template <class Pr, bool EDGE, bool LIN, bool COH = false>
+__device__ __forceinline__ void gather(const Params &P, const typename Pr::gs *g, const typename Pr::real *bnd,
                                        const double (*sev)[2], int x, int y, typename Pr::real inv,
                                        typename Pr::real f[9], typename Pr::real &gx, typename Pr::real &gy,
                                        typename Pr::real gsc) {
@@ -519,11 +583,11 @@ __device__ __forceinline__ void gather(const Params &P, const typename Pr::gs *_
   // the frame tiles, which lie within three nodes of a wall or of the end)
   if (!EDGE || (x >= 1 && x <= P.nx - 2 && y >= 1 && y <= P.ny - 2)) {
 #pragma unroll
-    for (int q = 0; q < 9; ++q) f[q] = gload(g, q * plane + idx - ex(q) - (ptrdiff_t)ey(q) * P.pitch, inv);
+    for (int q = 0; q < 9; ++q) f[q] = gld<COH>(g, q * plane + idx - ex(q) - (ptrdiff_t)ey(q) * P.pitch, inv);
 #pragma unroll
-    for (int q = 1; q < 9; ++q) g0[q] = gload(g, q * plane + idx, inv);
+    for (int q = 1; q < 9; ++q) g0[q] = gld<COH>(g, q * plane + idx, inv);
     g0[0] = 0;
-  } else if constexpr (sizeof(R) == 8) {
+  } else if constexpr (sizeof(R) == 8 && !COH) {
     // FP64: loads between the branches (the batched form below takes the
     // frame kernel past 128 registers, halving its blocks per SM)
     unsigned mask = 0;
@@ -538,13 +602,23 @@ __device__ __forceinline__ void gather(const Params &P, const typename Pr::gs *_
         f[q] = gload(g, q * plane + (size_t)sy * P.pitch + sx, inv);
       }
     }
-    if (mask) wall_rules<R, typename Pr::gs, LIN>(P, bnd, g, sev, x, y, g0, mask, f, gsc);
+    if (mask) {
+      int xw, yw;
+      R wn[4];
+      walls_of(P, x, y, xw, yw);
+      wall_n<COH>(P, bnd, xw, yw, x, y, wn);
+      wall_rules<R, typename Pr::gs, LIN, COH>(P, bnd, g, sev, x, y, xw, yw, wn, g0, mask, f, gsc);
+    }
   } else {
     // source of each population first (the node itself where the source
     // lies outside the lattice), then all eighteen loads without branches in
     // between, so that they are in flight together
     unsigned mask = 0;
     size_t src[9];
+    int xw, yw;
+    R wn[4];
+    walls_of(P, x, y, xw, yw);
+    if constexpr (COH) wall_n<COH>(P, bnd, xw, yw, x, y, wn);  // (in flight with the populations)
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
       int sx, sy;
@@ -554,13 +628,16 @@ __device__ __forceinline__ void gather(const Params &P, const typename Pr::gs *_
     }
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
-      g0[q] = gload(g, q * plane + idx, inv);
-      f[q] = gload(g, q * plane + src[q], inv);
+      g0[q] = gld<COH>(g, q * plane + idx, inv);
+      f[q] = gld<COH>(g, q * plane + src[q], inv);
     }
 #pragma unroll
     for (int q = 0; q < 9; ++q)
       if (mask & (1u << q)) f[q] = 0;
-    if (mask) wall_rules<R, typename Pr::gs, LIN>(P, bnd, g, sev, x, y, g0, mask, f, gsc);
+    if (mask) {
+      if constexpr (!COH) wall_n<COH>(P, bnd, xw, yw, x, y, wn);
+      wall_rules<R, typename Pr::gs, LIN, COH>(P, bnd, g, sev, x, y, xw, yw, wn, g0, mask, f, gsc);
+    }
   }
   first_moment(g0, gx, gy);
 }

@@ -62,6 +62,15 @@ struct StepPtrs {
                         //   device), or null: the frame tiles evaluate them
 };
 
+// Device pointers of one lattice for a resident launch: both buffers of each
+// state array, the barrier's two counters (zero between launches) and the
+// error flag.
+struct ResidentPtrs {
+  void *g[2], *u[2], *b[2];
+  unsigned *bar;
+  int *err;
+};
+
 struct TileShape {
   int tx, ty;
 };
@@ -109,6 +118,10 @@ struct Launchers {
   // last iteration of an odd count under a fused variant); one or two kernels
   cudaError_t (*step1)(const Params &p, const StepPtrs &s, cudaStream_t st);
   int (*kernels_per_step1)(const Params &p);
+  // n iterations in one cooperative launch, for the lattices where that is
+  // faster than launching every iteration (resident_applies)
+  bool (*resident_applies)(const Params &p);
+  cudaError_t (*resident)(const Params &p, const ResidentPtrs &s, int parity, int64_t k0, int n, cudaStream_t st);
   // TMA descriptors of one (g, u) buffer pair for a tile variant; returns
   // false if the variant does not use TMA.  out_g/out_u: CUtensorMap storage.
   bool (*tma_maps)(const Params &p, int variant, const void *g, const void *u, void *out_g, void *out_u);
@@ -181,6 +194,7 @@ struct lbs_handle {
   int64_t kdev_value;       // value held by *kdev (host mirror)
   int64_t unstable_at;
   int graph_chunk;
+  bool resident;            // runs of graph_chunk > 0 go out as resident launches
   cudaGraphExec_t graph[2];
   int graph_variant[2];
   size_t bytes;

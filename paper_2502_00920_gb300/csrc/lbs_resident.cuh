@@ -1,0 +1,398 @@
+// Resident iterations of liblbs: many iterations of a small lattice in one
+// cooperative launch.  Included by kernels_fp64.cu / kernels_fp32.cu /
+// kernels_fp16.cu after lbs_device.cuh.
+#pragma once
+#include "lbs_device.cuh"
+
+namespace lbs {
+
+// A tile of TX x TY nodes whose block has a thread for every node of the tile
+// plus its 2-node halo (R2): entry e < OWN is own node e, the rest are the ring.
+template <class Pr, int TX_, int TY_>
+struct ResCfg {
+  using PrT = Pr;
+  using real = typename Pr::real;
+  using us = typename Pr::us;
+  using gs = typename Pr::gs;
+  static constexpr int TX = TX_, TY = TY_;
+  static constexpr int R2W = TX + 4, R2H = TY + 4, R1W = TX + 2, R1H = TY + 2;
+  static constexpr int OWN = TX * TY, NRING = R2W * R2H - OWN;
+  static constexpr int NT = (R2W * R2H + 31) / 32 * 32;
+  static_assert(NT <= 1024, "one thread per node of R2");
+};
+
+// Barrier over the blocks of one cooperative launch: every block adds one to
+// *count, thread 0 polls until `target` arrivals (a bounded number of times:
+// false, with *err set, if they do not come).  The release of the arrival
+// covers the block's stores (ordered before it by the block barrier), the
+// acquire of the poll the reads that follow.
+constexpr uint32_t kMaxBarrierPolls = 1u << 22;
+__device__ __forceinline__ bool grid_barrier(unsigned *count, unsigned target, int *err) {
+  __syncthreads();
+  int ok = 1;
+  if (threadIdx.x == 0) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
+    ok = 0;
+    for (uint32_t i = 0; i < kMaxBarrierPolls; ++i) {
+      unsigned v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
+      if (v >= target) {
+        ok = 1;
+        break;
+      }
+    }
+    if (!ok) atomicExch(err, 1);
+  }
+  return __syncthreads_and(ok) != 0;
+}
+
+// keep a loop-invariant value in its register (the compiler otherwise
+// converts the double parameter again in every iteration)
+__device__ __forceinline__ float pinned(float v) {
+  asm volatile("" : "+f"(v));
+  return v;
+}
+__device__ __forceinline__ double pinned(double v) {
+  asm volatile("" : "+d"(v));
+  return v;
+}
+
+// The own-value wall rules of wall_rules() for one node with what does not
+// change between iterations taken out: sev holds the edges' values in the
+// compute type, js the momentum of a diagonal link between two Dirichlet walls
+// (their mean), and the sums leave out the terms whose factor e_a e_b is zero.
+template <class R>
+__device__ __forceinline__ void wall_rules_own(unsigned mask, unsigned crossx, unsigned crossy, bool dirx, bool diry,
+                                               R sgx, R sgy, R ics2, R cj, const R wn[4], const R *Tx, const R *Ty,
+                                               const R *js, const R g0[9], R f[9]) {
+  R r = 0, mxx = 0, mxy = 0, myy = 0;
+#pragma unroll
+  for (int q = 0; q < 9; ++q) {
+    r += g0[q];
+    if (ex(q) != 0) mxx += g0[q];
+    if (ex(q) * ey(q) != 0) mxy += R(ex(q) * ey(q)) * g0[q];
+    if (ey(q) != 0) myy += g0[q];
+  }
+  const R Axx_o = R(3) * mxx, Ayy_o = R(3) * myy;
+  const R Axx_x = (wn[0] - sgx * Tx[0]) * ics2, axy_x = (wn[1] - sgx * Tx[1]) * ics2;
+  const R Ayy_y = (wn[2] - sgy * Ty[1]) * ics2, axy_y = (wn[3] - sgy * Ty[0]) * ics2;
+#pragma unroll
+  for (int q = 1; q < 9; ++q) {
+    if (!(mask & (1u << q))) continue;
+    const bool ox = ex(q) != 0 && (crossx & (1u << q)), oy = ey(q) != 0 && (crossy & (1u << q));
+    const bool dxw = ox && dirx, dyw = oy && diry;
+    if (dxw || dyw) {
+      const R *j = dxw && dyw ? js : (dxw ? Tx : Ty);
+      f[q] = g0[opp(q)] + R(2) * wq<R>(q) * cj * (R(ex(q)) * j[0] + R(ey(q)) * j[1]);
+    } else {
+      const R Axx = ox ? Axx_x : Axx_o;
+      const R Ayy = oy ? Ayy_y : Ayy_o;
+      if (ex(q) * ey(q) == 0) {
+        f[q] = -g0[opp(q)] + wq<R>(q) * (R(4) * r - R(3) * r + R(3) * (ex(q) != 0 ? Axx : Ayy) - (Axx + Ayy));
+      } else {
+        const R Axy = (ox && oy) ? R(0.5) * (axy_x + axy_y) : (ox ? axy_x : axy_y);
+        const R eAe = Axx + R(2 * ex(q) * ey(q)) * Axy + Ayy;
+        f[q] = -g0[opp(q)] + wq<R>(q) * (R(4) * r - R(3) * r * R(2) + R(3) * eAe - (Axx + Ayy));
+      }
+    }
+  }
+}
+
+template <bool B, class X, class Y>
+struct Pick {
+  using type = X;
+};
+template <class X, class Y>
+struct Pick<false, X, Y> {
+  using type = Y;
+};
+
+// iterations whose edge values are evaluated at once
+constexpr int kSevBatch = 32;
+
+// n iterations from iteration k0 (buffers of `parity`) of the whole lattice,
+// one block per tile, a grid barrier between iterations.  The phases are those
+// of step_tile with every node's operations unchanged (the results are the
+// same bits), but what does not depend on the iteration is computed once: each
+// thread keeps its node's streaming sources, its finite-difference taps and
+// u(t) in registers (u on the halo is recomputed by every block that needs
+// it, so it never travels), and own nodes keep their g.  g and the walls' N go
+// through L2, both buffers in turn; u is stored by the last iteration.  The
+// barrier's counters are zero between launches: the last block to leave clears
+// them.  A launch that finds the error flag set does nothing.
+template <class C, bool LIN>
+__global__ void __launch_bounds__(C::NT) resident_kernel(const Params P, const ResidentPtrs S, int parity, int64_t k0,
+                                                         int n, int ntx) {
+  using gs = typename C::gs;
+  using us = typename C::us;
+  using R = typename C::real;
+  using T = typename Pick<LIN, double, R>::type;  // edge values: the linear reading takes them in double
+  __shared__ us su[C::R2H * C::R2W];
+  __shared__ R sn[4][C::R1H * C::R1W];
+  // per iteration: the four edges' values, then the four corners' means
+  __shared__ T sev[kSevBatch][8][2];
+  int bad = 0;
+  if (threadIdx.x == 0) bad = *(volatile int *)S.err;
+  if (__syncthreads_or(bad)) return;
+
+  const int x0 = (int)(blockIdx.x % ntx) * C::TX, y0 = (int)(blockIdx.x / ntx) * C::TY;
+  const int plane = P.ny * P.pitch;
+  const bool walls = !(P.per_x && P.per_y);
+  const R inv = pinned(gscale_inv<gs, R>(P)), scl = pinned(gscale<gs, R>(P));
+  const R kap = pinned((R)P.kappa * inv), idx_ = pinned((R)P.inv_dx);
+  const R lam = pinned((R)P.lam), mu = pinned((R)P.mu);
+  const CollideK<R> K = collide_k<R>(pinned((R)P.omega), pinned((R)P.sigma), scl);
+  const R sbx = pinned((R)(P.rho0 * P.body[0])), sby = pinned((R)(P.rho0 * P.body[1]));
+  const R ics2 = pinned((R)P.inv_cs2 * scl), cj = pinned((R)(P.c * P.inv_cs2) * scl);
+
+  // phase 1: this thread's node of R2
+  const int e = threadIdx.x;
+  int rx = 0, ry = 0, x = 0, y = 0, idx = 0, src[9], xw = -1, yw = -1;
+  bool in = false, own = false;
+  unsigned mask = 0, crossx = 0, crossy = 0;
+  us uu;
+  if (e < C::OWN + C::NRING) {
+    if (e < C::OWN) {
+      rx = e % C::TX + 2;
+      ry = e / C::TX + 2;
+    } else {
+      ring_pos<C>(e - C::OWN, rx, ry);
+    }
+    x = x0 - 2 + rx;
+    y = y0 - 2 + ry;
+    own = e < C::OWN && x < P.nx && y < P.ny;
+    in = locate(P, x, y);
+  }
+  const int us_at = ry * C::R2W + rx;
+  if (in) {
+    idx = y * P.pitch + x;
+    walls_of(P, x, y, xw, yw);
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+      int sx, sy;
+      bool ox, oy;
+      const bool inside = stream_source(P, x, y, q, sx, sy);
+      link_crosses(P, x, y, q, ox, oy);
+      if (!inside) mask |= 1u << q;
+      if (ox) crossx |= 1u << q;
+      if (oy) crossy |= 1u << q;
+      src[q] = q * plane + (inside ? sy * P.pitch + sx : idx);
+    }
+    uu = ld_coh((const us *)S.u[parity] + idx);
+  }
+  const bool nx_ = xw >= 0 && P.etype[xw] == LBS_NEUMANN, ny_ = yw >= 0 && P.etype[yw] == LBS_NEUMANN;
+  const int wx_at = nx_ ? (int)side_entry(P, 0, xw, y) : 0, wy_at = ny_ ? (int)side_entry(P, 0, yw, x) : 0;
+  const bool dirx = xw >= 0 && P.etype[xw] == LBS_DIRICHLET, diry = yw >= 0 && P.etype[yw] == LBS_DIRICHLET;
+  const R sgx = (xw == kRight) ? R(1) : R(-1), sgy = (yw == kTop) ? R(1) : R(-1);
+  const int corner = 4 + (xw == kRight ? 1 : 0) + (yw == kTop ? 2 : 0);
+
+  // phase 2: this thread's node of R1 and its taps of u
+  const int r1x = e % C::R1W, r1y = e / C::R1W;
+  int ux1 = 0, ux0 = 0, uy1 = 0, uy0 = 0, gx1 = x0 - 1 + r1x, gy1 = y0 - 1 + r1y;
+  bool in1 = e < C::R1W * C::R1H && locate(P, gx1, gy1), keep1 = false;
+  R sx1 = 0, sy1 = 0;
+  if (in1) {
+    int xa, xb, ya, yb;
+    bool onex, oney;
+    fd_taps<true>(P, r1x + 1, r1y + 1, gx1, gy1, xa, xb, ya, yb, onex, oney);
+    ux1 = (r1y + 1) * C::R2W + xa;
+    ux0 = (r1y + 1) * C::R2W + xb;
+    uy1 = ya * C::R2W + r1x + 1;
+    uy0 = yb * C::R2W + r1x + 1;
+    sx1 = onex ? idx_ : R(0.5) * idx_;
+    sy1 = oney ? idx_ : R(0.5) * idx_;
+    keep1 = r1_own_node<C>(P, x0, y0, r1x, r1y) && (on_wall(P, gx1, gy1) || (LIN && P.extrap));
+  }
+  // phase 3: the own node's taps of N
+  int nx1 = 0, nx0 = 0, ny1 = 0, ny0 = 0;
+  R sx2 = 0, sy2 = 0;
+  if (own) {
+    int xa, xb, ya, yb;
+    bool onex, oney;
+    fd_taps<true>(P, rx - 1, ry - 1, x, y, xa, xb, ya, yb, onex, oney);
+    nx1 = (ry - 1) * C::R1W + xa;
+    nx0 = (ry - 1) * C::R1W + xb;
+    ny1 = ya * C::R1W + rx - 1;
+    ny0 = yb * C::R1W + rx - 1;
+    sx2 = onex ? idx_ : R(0.5) * idx_;
+    sy2 = oney ? idx_ : R(0.5) * idx_;
+  }
+
+  R g0[9];
+  for (int it = 0; it < n; ++it) {
+    const int p = (parity + it) & 1;
+    const gs *g = (const gs *)S.g[p];
+    const R *bnd = (const R *)S.b[p];
+    R f[9], wn[4] = {R(0), R(0), R(0), R(0)};
+    if (in) {
+      if (nx_) {
+        wn[0] = ld_coh(bnd + wx_at);
+        wn[1] = ld_coh(bnd + wx_at + 2);
+      }
+      if (ny_) {
+        wn[2] = ld_coh(bnd + wy_at + 3);
+        wn[3] = ld_coh(bnd + wy_at + 1);
+      }
+#pragma unroll
+      for (int q = 0; q < 9; ++q) f[q] = half_wide(ld_coh(g + src[q]));
+      if (it == 0 || !own) {
+#pragma unroll
+        for (int q = 0; q < 9; ++q) g0[q] = half_wide(ld_coh(g + (q * plane + idx)));
+      }
+      if (mask) {
+#pragma unroll
+        for (int q = 0; q < 9; ++q)
+          if (mask & (1u << q)) f[q] = 0;
+      }
+    }
+    if (walls && it % kSevBatch == 0) {
+      // (while the populations are in flight)
+      for (int j = threadIdx.x; j < kSevBatch * 4; j += C::NT) {
+        double v[2];
+        if (it + j / 4 < n) {
+          edge_value(P, j % 4, k0 + it + j / 4, v);
+          sev[j / 4][j % 4][0] = (T)v[0];
+          sev[j / 4][j % 4][1] = (T)v[1];
+        }
+      }
+      if constexpr (!LIN) {
+        for (int j = threadIdx.x; j < kSevBatch * 4; j += C::NT) {
+          double a[2], b[2];
+          if (it + j / 4 < n && P.etype[kLeft + j % 2] == LBS_DIRICHLET &&
+              P.etype[kBottom + j % 4 / 2] == LBS_DIRICHLET) {
+            edge_value(P, kLeft + j % 2, k0 + it + j / 4, a);
+            edge_value(P, kBottom + j % 4 / 2, k0 + it + j / 4, b);
+            sev[j / 4][4 + j % 4][0] = (T)(0.5 * (a[0] + b[0]));
+            sev[j / 4][4 + j % 4][1] = (T)(0.5 * (a[1] + b[1]));
+          }
+        }
+      }
+      __syncthreads();
+    }
+    if (in) {
+      if (mask) {
+        const auto *ev = sev[it % kSevBatch];
+        if constexpr (LIN) {
+          R wnl[4];
+          wall_n<true>(P, bnd, xw, yw, x, y, wnl);
+          wall_rules<R, gs, true, true>(P, bnd, g, ev, x, y, xw, yw, wnl, g0, mask, f, scl);
+        } else {
+          wall_rules_own<R>(mask, crossx, crossy, dirx, diry, sgx, sgy, ics2, cj, wn, ev[xw < 0 ? 0 : xw],
+                            ev[yw < 0 ? 0 : yw], ev[corner], g0, f);
+        }
+      }
+      R gmx, gmy, fmx, fmy;
+      first_moment(g0, gmx, gmy);
+      first_moment(f, fmx, fmy);
+      uu = uadd_k(uu, kap, gmx + fmx, gmy + fmy);
+      su[us_at] = uu;
+    }
+    __syncthreads();
+    if (in1) {
+      R H[4], N[4], dxx, dxy, dyx, dyy;
+      udiff(su[ux1], su[ux0], dxx, dxy);
+      udiff(su[uy1], su[uy0], dyx, dyy);
+      H[0] = dxx * sx1;
+      H[1] = dyx * sy1;
+      H[2] = dxy * sx1;
+      H[3] = dyy * sy1;
+      material<R>(P, lam, mu, H, N);
+#pragma unroll
+      for (int m = 0; m < 4; ++m) sn[m][e] = N[m];
+      if (keep1) {
+        R *bo = (R *)S.b[p ^ 1];
+        if (on_wall(P, gx1, gy1)) store_wall_n<R>(P, bo, gx1, gy1, N);
+        if (LIN && P.extrap) store_inner_n<R>(P, bo, gx1, gy1, N);
+      }
+    }
+    __syncthreads();
+    if (own) {
+      const R Sx = fmr(sn[0][nx1] - sn[0][nx0], sx2, fmr(sn[1][ny1] - sn[1][ny0], sy2, sbx));
+      const R Sy = fmr(sn[2][nx1] - sn[2][nx0], sx2, fmr(sn[3][ny1] - sn[3][ny0], sy2, sby));
+      collide<R>(f, Sx, Sy, K);
+      gs *go = (gs *)S.g[p ^ 1];
+#pragma unroll
+      for (int q = 0; q < 9; ++q) {
+        gstore(go, (size_t)(q * plane + idx), f[q], scl);
+        if constexpr (sizeof(gs) == 2) g0[q] = __half2float(__float2half_rn(f[q]));
+        else g0[q] = f[q];
+      }
+    }
+    if (it + 1 < n && gridDim.x > 1) {
+      if (!grid_barrier(S.bar, (unsigned)(it + 1) * gridDim.x, S.err)) return;
+    } else {
+      __syncthreads();
+    }
+  }
+  if (own) ((us *)S.u[(parity + n) & 1])[idx] = uu;
+  if (gridDim.x > 1 && threadIdx.x == 0 && atomicAdd(&S.bar[1], 1u) == gridDim.x - 1) {
+    S.bar[0] = 0;
+    S.bar[1] = 0;
+  }
+}
+
+// blocks of a resident kernel that are on the GPU at once
+template <class C, bool LIN>
+int resident_capacity() {
+  static const int cap = [] {
+    int dev = 0, sms = 0, per = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, resident_kernel<C, LIN>, C::NT, 0);
+    return sms * per;
+  }();
+  return cap;
+}
+
+inline int resident_sms() {
+  static const int sms = [] {
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return n;
+  }();
+  return sms;
+}
+
+template <class C>
+int resident_tiles(const Params &P) {
+  const int64_t n = (int64_t)((P.nx + C::TX - 1) / C::TX) * ((P.ny + C::TY - 1) / C::TY);
+  return n < (1 << 20) ? (int)n : 1 << 20;
+}
+
+// The tile a lattice's resident launches run on: the small one while every
+// tile has an SM of its own, the large one while its tiles number at most
+// `large_most`, none (0) for larger lattices, which advance one iteration per
+// launch.  Small tiles have the shorter iteration, large ones reach further
+// and leave room for other lattices' launches (each shape's lines are
+// measured at the precisions' instantiations).
+enum { kResidentNone = 0, kResidentSmall = 1, kResidentLarge = 2 };
+template <class Small, class Large>
+int resident_shape(const Params &P, int large_most) {
+  const int cs = P.extrap ? resident_capacity<Small, true>() : resident_capacity<Small, false>();
+  const int cl = P.extrap ? resident_capacity<Large, true>() : resident_capacity<Large, false>();
+  const int ns = resident_tiles<Small>(P), nl = resident_tiles<Large>(P);
+  if (ns <= resident_sms() && ns <= cs) return kResidentSmall;
+  if (nl <= large_most && nl <= cl) return kResidentLarge;
+  return kResidentNone;
+}
+
+template <class C>
+cudaError_t launch_resident_c(const Params &P, const ResidentPtrs &S, int parity, int64_t k0, int n, cudaStream_t st) {
+  int ntx = (P.nx + C::TX - 1) / C::TX, nty = (P.ny + C::TY - 1) / C::TY;
+  void *args[] = {(void *)&P, (void *)&S, &parity, &k0, &n, &ntx};
+  const void *kernel = P.extrap ? (const void *)resident_kernel<C, true> : (const void *)resident_kernel<C, false>;
+  return cudaLaunchCooperativeKernel(kernel, dim3(ntx * nty), dim3(C::NT), args, 0, st);
+}
+
+template <class Small, class Large>
+cudaError_t launch_resident(const Params &P, const ResidentPtrs &S, int parity, int64_t k0, int n, int large_most,
+                            cudaStream_t st) {
+  switch (resident_shape<Small, Large>(P, large_most)) {
+    case kResidentSmall: return launch_resident_c<Small>(P, S, parity, k0, n, st);
+    case kResidentLarge: return launch_resident_c<Large>(P, S, parity, k0, n, st);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+}  // namespace lbs
