@@ -1,4 +1,6 @@
 // FP16 storage (scaled), FP32 arithmetic, u as a float pair: kernel instantiations and launchers of liblbs.
+#include <string.h>
+
 #include "lbs_device.cuh"
 #include "lbs_batch.cuh"
 #include "lbs_resident.cuh"
@@ -76,6 +78,11 @@ bool tma_maps(const Params &p, int v, const void *g, const void *u, void *og, vo
   return make_tma_maps<V4>(p, g, u, og, ou);
 }
 
+void coef(const Params &p, void *out) {
+  const auto k = make_coef<P::gs, P::real>(p);
+  memcpy(out, &k, sizeof(k));
+}
+
 // resident launches: the tiles and lines of single precision (us per iteration
 // on walled neo-Hooke lattices, one lattice alone / three side by side, against
 // launching every iteration from a graph: 40 x 40 10.1 / 3.5 -> 2.8 / 0.94,
@@ -112,6 +119,7 @@ const Launchers kL = {kVariants,
                       iterations_per_call,
                       launch_step<V0>,
                       step_kernel_count<V0>,
+                      coef,
                       resident_applies,
                       resident,
                       tma_maps,

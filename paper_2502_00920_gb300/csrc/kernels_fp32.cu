@@ -1,4 +1,6 @@
 // FP32 storage and arithmetic, u as a float pair: kernel instantiations and launchers of liblbs.
+#include <string.h>
+
 #include "lbs_device.cuh"
 #include "lbs_batch.cuh"
 #include "lbs_resident.cuh"
@@ -95,6 +97,11 @@ bool tma_maps(const Params &p, int v, const void *g, const void *u, void *og, vo
   return make_tma_maps<V4>(p, g, u, og, ou);
 }
 
+void coef(const Params &p, void *out) {
+  const auto k = make_coef<P::gs, P::real>(p);
+  memcpy(out, &k, sizeof(k));
+}
+
 // resident launches (us per iteration on walled neo-Hooke lattices, one lattice
 // alone / three advancing side by side; launching every iteration from a graph
 // before them): 32 x 32 9.1 / 3.1 -> 2.9 / 0.95 and 128 x 128 9.5 / 3.3 ->
@@ -135,6 +142,7 @@ const Launchers kL = {kVariants,
                       iterations_per_call,
                       launch_step<V0>,
                       step_kernel_count<V0>,
+                      coef,
                       resident_applies,
                       resident,
                       tma_maps,

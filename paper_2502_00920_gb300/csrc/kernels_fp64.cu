@@ -1,4 +1,6 @@
 // FP64 storage and arithmetic: kernel instantiations and launchers of liblbs.
+#include <string.h>
+
 #include "lbs_device.cuh"
 #include "lbs_batch.cuh"
 #include "lbs_resident.cuh"
@@ -58,6 +60,11 @@ bool tma_maps(const Params &p, int v, const void *g, const void *u, void *og, vo
   return make_tma_maps<V4>(p, g, u, og, ou);
 }
 
+void coef(const Params &p, void *out) {
+  const auto k = make_coef<P::gs, P::real>(p);
+  memcpy(out, &k, sizeof(k));
+}
+
 // resident launches (us per iteration on walled neo-Hooke lattices, one lattice
 // alone / three side by side, against launching every iteration from a graph):
 // 40 x 40 26.4 / 8.9 -> 9.2 / 3.1, 160 x 40 26.2 / 8.8 -> 9.0 / 4.2 and 96 x 96
@@ -98,6 +105,7 @@ const Launchers kL = {kVariants,
                       iterations_per_call,
                       launch_step<V0>,
                       step_kernel_count<V0>,
+                      coef,
                       resident_applies,
                       resident,
                       tma_maps,

@@ -20,10 +20,14 @@ __device__ __forceinline__ void batch_walk(const BatchLattice *lats, const Batch
                                            int *err) {
   using H = typename FrameCfg<C, SPLIT>::type;
   constexpr int parts = C::TY / H::TY;
+  using R = typename C::real;
   __shared__ Params sP;
+  __shared__ Coef<R> sC;
   __shared__ StepPtrs sS;
   __shared__ BatchTile sT;
   __shared__ int skip;
+  static_assert(sizeof(Coef<R>) / sizeof(R) <= 32 && sizeof(Coef<R>) <= sizeof(BatchLattice::coef),
+                "one lane copies each coefficient");
   static_assert(sizeof(Params) % 8 == 0, "the tile header is copied in 8-byte words");
   for (int t = blockIdx.x; t < ntiles * parts; t += gridDim.x) {
     // the tile's lattice header, read by the first warp: every lane reads the
@@ -36,6 +40,8 @@ __device__ __forceinline__ void batch_walk(const BatchLattice *lats, const Batch
       if (!sk)
         for (int w = threadIdx.x; w < (int)(sizeof(Params) / 8); w += 32)
           ((long long *)&sP)[w] = ((const long long *)&L.P)[w];
+      if (!sk && threadIdx.x < sizeof(Coef<R>) / sizeof(R))
+        ((R *)&sC)[threadIdx.x] = ((const R *)L.coef)[threadIdx.x];
       if (threadIdx.x == 0) {
         skip = sk;
         sT = T;
@@ -57,7 +63,7 @@ __device__ __forceinline__ void batch_walk(const BatchLattice *lats, const Batch
       }
     }
     __syncthreads();
-    if (!skip) step_tile<H, EDGE, LIN>(sP, sS, sT.a * C::TX, sT.b * C::TY + (t % parts) * H::TY);
+    if (!skip) step_tile<H, EDGE, LIN>(sP, sC, sS, sT.a * C::TX, sT.b * C::TY + (t % parts) * H::TY);
     __syncthreads();  // the next tile reuses the shared memory
   }
 }

@@ -324,11 +324,10 @@ __device__ __forceinline__ void wall_n(const Params &P, const R *bnd, int xw, in
 
 template <class R, class G, bool LIN, bool COH>
 __device__ void wall_rules(const Params &P, const R *bnd, const G *g, const double (*sev)[2], int x, int y, int xw,
-                           int yw, const R wn[4], const R g0[9], unsigned mask, R f[9], R gsc) {
+                           int yw, const R wn[4], const R g0[9], unsigned mask, R f[9], R ics2, R cj) {
   const bool xn = xw >= 0 && P.etype[xw] == LBS_NEUMANN;
   const bool yn = yw >= 0 && P.etype[yw] == LBS_NEUMANN;
-  // Pi*/cs^2 from N and T* is brought into the units of g (times gsc)
-  const R ics2 = (R)P.inv_cs2 * gsc;
+  // (ics2 brings Pi*/cs^2 from N and T* into the units of g)
   // own moments (collision leaves r and Pi unchanged): r, A = Pi / cs^2 = 3 sum e e g
   R r = 0, mxx = 0, mxy = 0, myy = 0;
 #pragma unroll
@@ -400,7 +399,6 @@ __device__ void wall_rules(const Params &P, const R *bnd, const G *g, const doub
       }
     }
   }
-  const R cj = (R)(P.c * P.inv_cs2) * gsc;
 #pragma unroll
   for (int q = 1; q < 9; ++q) {
     if (!(mask & (1u << q))) continue;
@@ -473,7 +471,7 @@ struct CollideK {
   R mo, m6, m9, m12, a1, a5, s9, s36;
 };
 template <class R>
-__device__ __forceinline__ CollideK<R> collide_k(R omega, R sigma, R scl) {
+__host__ __device__ __forceinline__ CollideK<R> collide_k(R omega, R sigma, R scl) {
   const R ss = sigma * scl;
   return {-omega,
           -omega * (R(1) / R(6)),
@@ -548,6 +546,39 @@ __device__ __forceinline__ void collide(R f[9], R Sx, R Sy, const CollideK<R> &K
   }
 }
 
+// The coefficients of the scheme in the compute type, evaluated on the host
+// once per launch and handed to the kernels beside Params.  (Evaluated in the
+// kernels, the conversions from the double parameters and the products cost
+// every thread some twenty FP64 instructions, which GB300 issues at a few per
+// cent of the FP32 rate; a thread updates only two to four nodes.)
+template <class R>
+struct Coef {
+  R inv, scl;    // 2^-gshift, 2^gshift: storage units of g
+  R kap;         // displacement increment per unit first moment
+  R lam, mu;
+  R idx, hdx;    // 1 / dx, 1 / (2 dx)
+  R sbx, sby;    // rho0 b
+  R ics2, cj;    // 1 / cs^2 and c / cs^2 in storage units of g (wall rules)
+  CollideK<R> K;
+};
+template <class G, class R>
+__host__ __device__ inline Coef<R> make_coef(const Params &P) {
+  Coef<R> k;
+  k.inv = gscale_inv<G, R>(P);
+  k.scl = gscale<G, R>(P);
+  k.kap = (R)P.kappa * k.inv;
+  k.lam = (R)P.lam;
+  k.mu = (R)P.mu;
+  k.idx = (R)P.inv_dx;
+  k.hdx = R(0.5) * k.idx;
+  k.sbx = (R)(P.rho0 * P.body[0]);
+  k.sby = (R)(P.rho0 * P.body[1]);
+  k.ics2 = (R)P.inv_cs2 * k.scl;
+  k.cj = (R)(P.c * P.inv_cs2) * k.scl;
+  k.K = collide_k<R>((R)P.omega, (R)P.sigma, k.scl);
+  return k;
+}
+
 // ------------------------------------------------------------------ tiles
 // A thread block owns a TX x TY tile of nodes; NTY thread rows, each thread
 // handles CPT = TY / NTY nodes of one column.  Shared memory holds u_{k+1}
@@ -571,12 +602,12 @@ struct TileCfg : TileGeom<TX_, TY_, NTY_> {
 // LIN: the two-point wall extrapolation (lattices with P.extrap set).
 template <class Pr, bool EDGE, bool LIN, bool COH = false>
 __device__ __forceinline__ void gather(const Params &P, const typename Pr::gs *g, const typename Pr::real *bnd,
-                                       const double (*sev)[2], int x, int y, typename Pr::real inv,
-                                       typename Pr::real f[9], typename Pr::real &gx, typename Pr::real &gy,
-                                       typename Pr::real gsc) {
+                                       const double (*sev)[2], int x, int y, const Coef<typename Pr::real> &k,
+                                       typename Pr::real f[9], typename Pr::real &gx, typename Pr::real &gy) {
   using R = typename Pr::real;
   const size_t plane = (size_t)P.ny * P.pitch;
   const size_t idx = (size_t)y * P.pitch + x;
+  const R inv = k.inv;
   R g0[9];
   // every streaming source inside the lattice without wrapping: loads at
   // fixed offsets, no boundary rule (all interior tiles, and most nodes of
@@ -607,7 +638,7 @@ __device__ __forceinline__ void gather(const Params &P, const typename Pr::gs *g
       R wn[4];
       walls_of(P, x, y, xw, yw);
       wall_n<COH>(P, bnd, xw, yw, x, y, wn);
-      wall_rules<R, typename Pr::gs, LIN, COH>(P, bnd, g, sev, x, y, xw, yw, wn, g0, mask, f, gsc);
+      wall_rules<R, typename Pr::gs, LIN, COH>(P, bnd, g, sev, x, y, xw, yw, wn, g0, mask, f, k.ics2, k.cj);
     }
   } else {
     // source of each population first (the node itself where the source
@@ -636,7 +667,7 @@ __device__ __forceinline__ void gather(const Params &P, const typename Pr::gs *g
       if (mask & (1u << q)) f[q] = 0;
     if (mask) {
       if constexpr (!COH) wall_n<COH>(P, bnd, xw, yw, x, y, wn);
-      wall_rules<R, typename Pr::gs, LIN, COH>(P, bnd, g, sev, x, y, xw, yw, wn, g0, mask, f, gsc);
+      wall_rules<R, typename Pr::gs, LIN, COH>(P, bnd, g, sev, x, y, xw, yw, wn, g0, mask, f, k.ics2, k.cj);
     }
   }
   first_moment(g0, gx, gy);
@@ -707,16 +738,16 @@ struct Fd {
 // to the side array (and, with LIN on a lattice with P.extrap set, N of the
 // nodes one step inwards to its second layer)
 template <class C, bool EDGE, bool LIN = false>
-__device__ __forceinline__ void phase_n(typename C::Smem &sm, const Params &P, int x0, int y0, typename C::real *bnd_out) {
+__device__ __forceinline__ void phase_n(typename C::Smem &sm, const Params &P, const Coef<typename C::real> &k, int x0,
+                                        int y0, typename C::real *bnd_out) {
   using R = typename C::real;
-  const R lam = (R)P.lam, mu = (R)P.mu, idx_ = (R)P.inv_dx;
   for (int e = threadIdx.x; e < C::R1W * C::R1H; e += C::NT) {
     const int rx = e % C::R1W, ry = e / C::R1W;
     int gx = x0 - 1 + rx, gy = y0 - 1 + ry;
     if (EDGE && !locate(P, gx, gy)) continue;
     R H[4], N[4];
-    Fd<C, EDGE>::grad(sm, P, rx, ry, gx, gy, idx_, H);
-    material<R>(P, lam, mu, H, N);
+    Fd<C, EDGE>::grad(sm, P, rx, ry, gx, gy, k.idx, H);
+    material<R>(P, k.lam, k.mu, H, N);
 #pragma unroll
     for (int m = 0; m < 4; ++m) sm.n[m][ry][rx] = N[m];
     if (EDGE && bnd_out && r1_own_node<C>(P, x0, y0, rx, ry)) {
@@ -728,7 +759,8 @@ __device__ __forceinline__ void phase_n(typename C::Smem &sm, const Params &P, i
 
 // The fused iteration on one tile.
 template <class C, bool EDGE, bool LIN = false>
-__device__ __forceinline__ void step_tile(const Params &P, const StepPtrs &S, int x0, int y0) {
+__device__ __forceinline__ void step_tile(const Params &P, const Coef<typename C::real> &c, const StepPtrs &S, int x0,
+                                          int y0) {
   using Pr_real = typename C::real;
   using R = Pr_real;
   using us = typename C::us;
@@ -751,9 +783,6 @@ __device__ __forceinline__ void step_tile(const Params &P, const StepPtrs &S, in
     }
     __syncthreads();
   }
-  // g is held in units of g * 2^gshift (1 unless FP16 storage)
-  const R inv = gscale_inv<typename C::gs, R>(P), scl = gscale<typename C::gs, R>(P);
-  const R kap = (R)P.kappa * inv;
   const int tx = threadIdx.x % C::TX, ty = threadIdx.x / C::TX;
 
   // phase 1a: own nodes (keep the streamed populations).  In a tile that
@@ -767,10 +796,10 @@ __device__ __forceinline__ void step_tile(const Params &P, const StepPtrs &S, in
     int x = x0 + lx, y = y0 + ly;
     if (EDGE && !locate(P, x, y)) continue;
     R gxm, gym;
-    gather<typename C::PrT, EDGE, LIN>(P, g, bnd, sev, x, y, inv, f[i], gxm, gym, scl);
+    gather<typename C::PrT, EDGE, LIN>(P, g, bnd, sev, x, y, c, f[i], gxm, gym);
     R fx, fy;
     first_moment(f[i], fx, fy);
-    sm.u[ly + 2][lx + 2] = uadd_k(u[(size_t)y * P.pitch + x], kap, gxm + fx, gym + fy);
+    sm.u[ly + 2][lx + 2] = uadd_k(u[(size_t)y * P.pitch + x], c.kap, gxm + fx, gym + fy);
   }
   // phase 1b: the 2-node frame (u only)
   for (int e = threadIdx.x; e < C::NRING; e += C::NT) {
@@ -779,30 +808,27 @@ __device__ __forceinline__ void step_tile(const Params &P, const StepPtrs &S, in
     int x = x0 - 2 + rx, y = y0 - 2 + ry;
     if (EDGE && !locate(P, x, y)) continue;
     R ff[9], gxm, gym;
-    gather<typename C::PrT, EDGE, LIN>(P, g, bnd, sev, x, y, inv, ff, gxm, gym, scl);
+    gather<typename C::PrT, EDGE, LIN>(P, g, bnd, sev, x, y, c, ff, gxm, gym);
     R fx, fy;
     first_moment(ff, fx, fy);
-    sm.u[ry][rx] = uadd_k(u[(size_t)y * P.pitch + x], kap, gxm + fx, gym + fy);
+    sm.u[ry][rx] = uadd_k(u[(size_t)y * P.pitch + x], c.kap, gxm + fx, gym + fy);
   }
   __syncthreads();
-  phase_n<C, EDGE, LIN>(sm, P, x0, y0, (R *)S.b_out);
+  phase_n<C, EDGE, LIN>(sm, P, c, x0, y0, (R *)S.b_out);
   __syncthreads();
   // phase 3: source, collision, store
   const size_t plane = (size_t)P.ny * P.pitch;
-  const R idx_ = (R)P.inv_dx;
-  const CollideK<R> K = collide_k<R>((R)P.omega, (R)P.sigma, scl);
-  const R sbx = (R)(P.rho0 * P.body[0]), sby = (R)(P.rho0 * P.body[1]);
 #pragma unroll
   for (int i = 0; i < C::CPT; ++i) {
     const int lx = tx, ly = ty + i * C::NTY;
     const int x = x0 + lx, y = y0 + ly;
     if (EDGE && (x >= P.nx || y >= P.ny)) continue;
     R Sx, Sy;
-    Fd<C, EDGE>::div(sm, P, lx + 1, ly + 1, x, y, idx_, sbx, sby, Sx, Sy);
-    collide<R>(f[i], Sx, Sy, K);
+    Fd<C, EDGE>::div(sm, P, lx + 1, ly + 1, x, y, c.idx, c.sbx, c.sby, Sx, Sy);
+    collide<R>(f[i], Sx, Sy, c.K);
     const size_t idx = (size_t)y * P.pitch + x;
 #pragma unroll
-    for (int q = 0; q < 9; ++q) gstore(go, q * plane + idx, f[i][q], scl);
+    for (int q = 0; q < 9; ++q) gstore(go, q * plane + idx, f[i][q], c.scl);
     uo[idx] = sm.u[ly + 2][lx + 2];
   }
 }
@@ -814,8 +840,9 @@ struct Cfg : TileCfg<Pr, TX, TY, NTY> {
 
 // interior tiles: R2 and its streaming sources lie inside, no wall, no wrap
 template <class C>
-__global__ void __launch_bounds__(C::NT) step_interior_kernel(const Params P, const StepPtrs S, int a_lo, int b_lo) {
-  step_tile<C, false>(P, S, (a_lo + blockIdx.x) * C::TX, (b_lo + blockIdx.y) * C::TY);
+__global__ void __launch_bounds__(C::NT) step_interior_kernel(const Params P, const Coef<typename C::real> c,
+                                                              const StepPtrs S, int a_lo, int b_lo) {
+  step_tile<C, false>(P, c, S, (a_lo + blockIdx.x) * C::TX, (b_lo + blockIdx.y) * C::TY);
 }
 
 // tiles of the frame around the interior block (walls, wrap, partial tiles):
@@ -836,14 +863,15 @@ struct FrameCfg<C, true> {
 };
 
 template <class C, bool LIN, bool SPLIT = false>
-__global__ void __launch_bounds__(FrameCfg<C, SPLIT>::type::NT) step_edge_kernel(const Params P, const StepPtrs S,
-                                                                                 int ntx, int a_lo, int a_hi,
+__global__ void __launch_bounds__(FrameCfg<C, SPLIT>::type::NT) step_edge_kernel(const Params P,
+                                                                                 const Coef<typename C::real> c,
+                                                                                 const StepPtrs S, int ntx, int a_lo, int a_hi,
                                                                                  int b_lo, int b_hi) {
   using H = typename FrameCfg<C, SPLIT>::type;
   constexpr int parts = C::TY / H::TY;
   int a, b;
   edge_tile(blockIdx.x / parts, ntx, a_lo, a_hi, b_lo, b_hi, a, b);
-  step_tile<H, true, LIN>(P, S, a * C::TX, b * C::TY + (blockIdx.x % parts) * H::TY);
+  step_tile<H, true, LIN>(P, c, S, a * C::TX, b * C::TY + (blockIdx.x % parts) * H::TY);
 }
 
 // the frame tiles of one iteration; the two-point wall extrapolation has its
@@ -852,6 +880,7 @@ template <class C>
 void launch_edge(const Params &P, const StepPtrs &S, int nedge, int ntx, int a_lo, int a_hi, int b_lo, int b_hi,
                  cudaStream_t st) {
   if (nedge <= 0) return;
+  const auto c = make_coef<typename C::gs, typename C::real>(P);
   if constexpr (C::CPT >= 2) {
     static const int sms = [] {
       int dev = 0, n = 0;
@@ -862,13 +891,13 @@ void launch_edge(const Params &P, const StepPtrs &S, int nedge, int ntx, int a_l
     if (nedge <= sms) {
       using H = typename FrameCfg<C, true>::type;
       const int nb = C::CPT * nedge;
-      if (P.extrap) step_edge_kernel<C, true, true><<<nb, H::NT, 0, st>>>(P, S, ntx, a_lo, a_hi, b_lo, b_hi);
-      else step_edge_kernel<C, false, true><<<nb, H::NT, 0, st>>>(P, S, ntx, a_lo, a_hi, b_lo, b_hi);
+      if (P.extrap) step_edge_kernel<C, true, true><<<nb, H::NT, 0, st>>>(P, c, S, ntx, a_lo, a_hi, b_lo, b_hi);
+      else step_edge_kernel<C, false, true><<<nb, H::NT, 0, st>>>(P, c, S, ntx, a_lo, a_hi, b_lo, b_hi);
       return;
     }
   }
-  if (P.extrap) step_edge_kernel<C, true><<<nedge, C::NT, 0, st>>>(P, S, ntx, a_lo, a_hi, b_lo, b_hi);
-  else step_edge_kernel<C, false><<<nedge, C::NT, 0, st>>>(P, S, ntx, a_lo, a_hi, b_lo, b_hi);
+  if (P.extrap) step_edge_kernel<C, true><<<nedge, C::NT, 0, st>>>(P, c, S, ntx, a_lo, a_hi, b_lo, b_hi);
+  else step_edge_kernel<C, false><<<nedge, C::NT, 0, st>>>(P, c, S, ntx, a_lo, a_hi, b_lo, b_hi);
 }
 
 // longest walk (tiles per persistent block) beside which a frame kernel runs
@@ -909,7 +938,8 @@ cudaError_t launch_step(const Params &P, const StepPtrs &S, cudaStream_t st) {
   const int nedge = ntx * nty - ni * nj;
   const bool beside = fork_begin(S, st, ni > 0 && nj > 0 && nedge > 0);
   if (beside) launch_edge<C>(P, S, nedge, ntx, a_lo, a_hi, b_lo, b_hi, S.fork->side);
-  if (ni > 0 && nj > 0) step_interior_kernel<C><<<dim3(ni, nj), C::NT, 0, st>>>(P, S, a_lo, b_lo);
+  if (ni > 0 && nj > 0) step_interior_kernel<C><<<dim3(ni, nj), C::NT, 0, st>>>(P, make_coef<typename C::gs, typename C::real>(P), S,
+                                                                                 a_lo, b_lo);
   if (!beside) launch_edge<C>(P, S, nedge, ntx, a_lo, a_hi, b_lo, b_hi, st);
   fork_end(S, st, beside);
   return cudaGetLastError();
@@ -995,17 +1025,14 @@ struct TmaCfg : TmaGeom<C::TX, C::TY, (int)sizeof(typename C::gs), (int)sizeof(t
 // entries into registers and keeps its own nodes' u for the store, and the
 // entries are written once all threads have read their u taps.
 template <class C>
-__device__ __forceinline__ void tma_tile(const Params &P, const StepPtrs &S, const typename C::gs *sg,
-                                         typename C::us *su, typename C::real *snb, int x0, int y0) {
+__device__ __forceinline__ void tma_tile(const Params &P, const Coef<typename C::real> &c, const StepPtrs &S,
+                                         const typename C::gs *sg, typename C::us *su, typename C::real *snb, int x0, int y0) {
   using T = TmaCfg<C>;
   using R = typename C::real;
   using us = typename C::us;
   using gs = typename C::gs;
-  // g is held in units of g * 2^gshift (1 unless FP16 storage)
-  const R inv = gscale_inv<gs, R>(P), scl = gscale<gs, R>(P);
-  const R kap = (R)P.kappa * inv;
-  auto G = [&](int q, int r, int c) -> R {
-    const gs v = sg[((size_t)q * T::GH + r) * T::GW + c];
+  auto G = [&](int q, int r, int col) -> R {
+    const gs v = sg[((size_t)q * T::GH + r) * T::GW + col];
     if constexpr (sizeof(gs) == 2) return __half2float(v);
     else return (R)v;
   };
@@ -1024,34 +1051,33 @@ __device__ __forceinline__ void tma_tile(const Params &P, const StepPtrs &S, con
     R gx, gy, fx, fy;
     first_moment(o, gx, gy);
     first_moment(p, fx, fy);
-    su[e] = uadd_k(su[e], kap, gx + fx, gy + fy);
+    su[e] = uadd_k(su[e], c.kap, gx + fx, gy + fy);
   }
   __syncthreads();
   // phase 2: N on R1
   constexpr int W1 = C::TX + 2, H1 = C::TY + 2, NE = W1 * H1, NPER = (NE + C::NT - 1) / C::NT;
   const int tx = threadIdx.x % C::TX, ty = threadIdx.x / C::TX;
-  const R hdx = R(0.5) * (R)P.inv_dx;
+  const R hdx = c.hdx;
   // own nodes' u(t+dt), read before N may overwrite the box
   us uown[C::CPT];
 #pragma unroll
   for (int i = 0; i < C::CPT; ++i) uown[i] = su[(ty + i * C::NTY + 2) * T::UW + (tx + 2)];
   {
-    const R lam = (R)P.lam, mu = (R)P.mu;
     R nreg[T::N_IN_U ? NPER : 1][4];
 #pragma unroll
     for (int k = 0; k < NPER; ++k) {
       const int e = threadIdx.x + k * C::NT;
       if (e >= NE) break;
       const int rx = e % W1, ry = e / W1;
-      const int c = (ry + 1) * T::UW + (rx + 1);
+      const int at = (ry + 1) * T::UW + (rx + 1);
       R dxx, dxy, dyx, dyy, H[4], N[4];
-      udiff(su[c + 1], su[c - 1], dxx, dxy);
-      udiff(su[c + T::UW], su[c - T::UW], dyx, dyy);
+      udiff(su[at + 1], su[at - 1], dxx, dxy);
+      udiff(su[at + T::UW], su[at - T::UW], dyx, dyy);
       H[0] = dxx * hdx;
       H[1] = dyx * hdx;
       H[2] = dxy * hdx;
       H[3] = dyy * hdx;
-      material<R>(P, lam, mu, H, N);
+      material<R>(P, c.lam, c.mu, H, N);
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
         if constexpr (T::N_IN_U) nreg[k][m] = N[m];
@@ -1073,8 +1099,7 @@ __device__ __forceinline__ void tma_tile(const Params &P, const StepPtrs &S, con
   __syncthreads();
   // phase 3: stream again from shared memory, source, collision, store
   const size_t plane = (size_t)P.ny * P.pitch;
-  const CollideK<R> K = collide_k<R>((R)P.omega, (R)P.sigma, scl);
-  const R sbx = (R)(P.rho0 * P.body[0]), sby = (R)(P.rho0 * P.body[1]);
+  const R sbx = c.sbx, sby = c.sby;
   gs *__restrict__ go = (gs *)S.g_out;
   us *__restrict__ uo = (us *)S.u_out;
 #pragma unroll
@@ -1088,16 +1113,17 @@ __device__ __forceinline__ void tma_tile(const Params &P, const StepPtrs &S, con
     auto n = [&](int m, int yy, int xx) -> R { return snb[(m * H1 + yy) * W1 + xx]; };
     const R Sx = fmr(n(0, ry, rx + 1) - n(0, ry, rx - 1), hdx, fmr(n(1, ry + 1, rx) - n(1, ry - 1, rx), hdx, sbx));
     const R Sy = fmr(n(2, ry, rx + 1) - n(2, ry, rx - 1), hdx, fmr(n(3, ry + 1, rx) - n(3, ry - 1, rx), hdx, sby));
-    collide<R>(f, Sx, Sy, K);
+    collide<R>(f, Sx, Sy, c.K);
     const size_t idx = (size_t)(y0 + ly) * P.pitch + (x0 + lx);
 #pragma unroll
-    for (int q = 0; q < 9; ++q) gstore(go, q * plane + idx, f[q], scl);
+    for (int q = 0; q < 9; ++q) gstore(go, q * plane + idx, f[q], c.scl);
     uo[idx] = uown[i];
   }
 }
 
 template <class C>
-__global__ void __launch_bounds__(C::NT) step_tma_kernel(const Params P, const StepPtrs S,
+__global__ void __launch_bounds__(C::NT) step_tma_kernel(const Params P, const Coef<typename C::real> c,
+                                                         const StepPtrs S,
                                                          const __grid_constant__ CUtensorMap tm_g,
                                                          const __grid_constant__ CUtensorMap tm_u, int a_lo, int b_lo) {
   using T = TmaCfg<C>;
@@ -1131,7 +1157,7 @@ __global__ void __launch_bounds__(C::NT) step_tma_kernel(const Params P, const S
     return;
   }
 
-  tma_tile<C>(P, S, sg, su, snb, x0, y0);
+  tma_tile<C>(P, c, S, sg, su, snb, x0, y0);
 }
 
 template <class C>
@@ -1146,7 +1172,8 @@ cudaError_t launch_step_tma(const Params &P, const StepPtrs &S, cudaStream_t st)
   const bool beside = fork_begin(S, st, ni > 0 && nj > 0 && nedge > 0);
   if (beside) launch_edge<C>(P, S, nedge, ntx, a_lo, a_hi, b_lo, b_hi, S.fork->side);
   if (ni > 0 && nj > 0)
-    step_tma_kernel<C><<<dim3(ni, nj), C::NT, T::SMEM, st>>>(P, S, *(const CUtensorMap *)S.tm_g,
+    step_tma_kernel<C><<<dim3(ni, nj), C::NT, T::SMEM, st>>>(P, make_coef<typename C::gs, typename C::real>(P), S,
+                                                               *(const CUtensorMap *)S.tm_g,
                                                                *(const CUtensorMap *)S.tm_u, a_lo, b_lo);
   if (!beside) launch_edge<C>(P, S, nedge, ntx, a_lo, a_hi, b_lo, b_hi, st);
   fork_end(S, st, beside);
@@ -1179,7 +1206,8 @@ __device__ __forceinline__ void tma2_issue(unsigned char *stage, uint64_t *bar, 
 }
 
 template <class C>
-__global__ void __launch_bounds__(C::NT) step_tma2_kernel(const Params P, const StepPtrs S,
+__global__ void __launch_bounds__(C::NT) step_tma2_kernel(const Params P, const Coef<typename C::real> c,
+                                                          const StepPtrs S,
                                                           const __grid_constant__ CUtensorMap tm_g,
                                                           const __grid_constant__ CUtensorMap tm_u, int a_lo, int b_lo,
                                                           int ni, int ntiles) {
@@ -1239,7 +1267,7 @@ __global__ void __launch_bounds__(C::NT) step_tma2_kernel(const Params P, const 
     }
     int x0, y0;
     tile_xy(t, x0, y0);
-    tma_tile<C>(P, S, sg, su, T::N_IN_U ? (R *)su : (R *)(dsm + T2::OFF_N), x0, y0);
+    tma_tile<C>(P, c, S, sg, su, T::N_IN_U ? (R *)su : (R *)(dsm + T2::OFF_N), x0, y0);
     __syncthreads();  // this stage is free for the prefetch after next
   }
 }
@@ -1271,7 +1299,8 @@ cudaError_t launch_step_tma2(const Params &P, const StepPtrs &S, cudaStream_t st
   if (beside) launch_edge<C>(P, S, nedge, ntx, a_lo, a_hi, b_lo, b_hi, S.fork->side);
   if (ni > 0 && nj > 0) {
     step_tma2_kernel<C><<<ntiles < blocks ? ntiles : blocks, C::NT, T2::SMEM, st>>>(
-        P, S, *(const CUtensorMap *)S.tm_g, *(const CUtensorMap *)S.tm_u, a_lo, b_lo, ni, ntiles);
+        P, make_coef<typename C::gs, typename C::real>(P), S, *(const CUtensorMap *)S.tm_g,
+        *(const CUtensorMap *)S.tm_u, a_lo, b_lo, ni, ntiles);
   }
   if (!beside) launch_edge<C>(P, S, nedge, ntx, a_lo, a_hi, b_lo, b_hi, st);
   fork_end(S, st, beside);
@@ -1323,18 +1352,14 @@ __device__ __forceinline__ typename G::gs fstore(typename G::real v) {
 // both iterations of one tile from its staged boxes; stores the nodes of the
 // tile that lie in the lattice
 template <class C>
-__device__ __forceinline__ void fused2_tile(const Params &P, const StepPtrs &S, const typename C::gs *sg,
-                                            typename C::us *su, typename C::gs *sh, typename C::real *sn, int x0,
+__device__ __forceinline__ void fused2_tile(const Params &P, const Coef<typename C::real> &c, const StepPtrs &S,
+                                            const typename C::gs *sg, typename C::us *su, typename C::gs *sh, typename C::real *sn, int x0,
                                             int y0) {
   using F = Fuse2Cfg<C>;
   using R = typename C::real;
   using us = typename C::us;
   using gs = typename C::gs;
-  const R inv = gscale_inv<gs, R>(P), scl = gscale<gs, R>(P);
-  const R kap = (R)P.kappa * inv, hdx = R(0.5) * (R)P.inv_dx;
-  const R lam = (R)P.lam, mu = (R)P.mu;
-  const CollideK<R> K = collide_k<R>((R)P.omega, (R)P.sigma, scl);
-  const R sbx = (R)(P.rho0 * P.body[0]), sby = (R)(P.rho0 * P.body[1]);
+  const R hdx = c.hdx, sbx = c.sbx, sby = c.sby;
   // u(t+dt) at node offset (i, j) from the populations of array A (g box or g1)
   auto advance_u = [&](auto A, int i, int j) {
     R p[9], o[9];
@@ -1347,7 +1372,7 @@ __device__ __forceinline__ void fused2_tile(const Params &P, const StepPtrs &S, 
     first_moment(o, gx, gy);
     first_moment(p, fx, fy);
     us &uu = su[F::u(i, j)];
-    uu = uadd_k(uu, kap, gx + fx, gy + fy);
+    uu = uadd_k(uu, c.kap, gx + fx, gy + fy);
   };
   // N at node offset (i, j) from u in the u box
   auto stress = [&](int i, int j) {
@@ -1358,7 +1383,7 @@ __device__ __forceinline__ void fused2_tile(const Params &P, const StepPtrs &S, 
     H[1] = dyx * hdx;
     H[2] = dxy * hdx;
     H[3] = dyy * hdx;
-    material<R>(P, lam, mu, H, N);
+    material<R>(P, c.lam, c.mu, H, N);
 #pragma unroll
     for (int m = 0; m < 4; ++m) sn[F::n(m, i, j)] = N[m];
   };
@@ -1369,7 +1394,7 @@ __device__ __forceinline__ void fused2_tile(const Params &P, const StepPtrs &S, 
     auto n = [&](int m, int ii, int jj) -> R { return sn[F::n(m, ii, jj)]; };
     const R Sx = fmr(n(0, i + 1, j) - n(0, i - 1, j), hdx, fmr(n(1, i, j + 1) - n(1, i, j - 1), hdx, sbx));
     const R Sy = fmr(n(2, i + 1, j) - n(2, i - 1, j), hdx, fmr(n(3, i, j + 1) - n(3, i, j - 1), hdx, sby));
-    collide<R>(f, Sx, Sy, K);
+    collide<R>(f, Sx, Sy, c.K);
   };
   auto Gk = [&](int q, int i, int j) -> R { return fconv<F>(sg[F::g(q, i, j)]); };
   auto G1 = [&](int q, int i, int j) -> R { return fconv<F>(sh[F::h(q, i, j)]); };
@@ -1398,21 +1423,22 @@ __device__ __forceinline__ void fused2_tile(const Params &P, const StepPtrs &S, 
   us *__restrict__ uo = (us *)S.u_out;
   const int tx = threadIdx.x % C::TX, ty = threadIdx.x / C::TX;
 #pragma unroll
-  for (int c = 0; c < C::CPT; ++c) {
-    const int i = tx, j = ty + c * C::NTY;
+  for (int m = 0; m < C::CPT; ++m) {
+    const int i = tx, j = ty + m * C::NTY;
     R f[9];
     collide_at(G1, i, j, f);
     const int x = x0 + i, y = y0 + j;
     if (x >= P.nx || y >= P.ny) continue;
     const size_t idx = (size_t)y * P.pitch + x;
 #pragma unroll
-    for (int q = 0; q < 9; ++q) gstore(go, q * plane + idx, f[q], scl);
+    for (int q = 0; q < 9; ++q) gstore(go, q * plane + idx, f[q], c.scl);
     uo[idx] = su[F::u(i, j)];
   }
 }
 
 template <class C>
-__global__ void __launch_bounds__(C::NT) step_fused2_tma_kernel(const Params P, const StepPtrs S,
+__global__ void __launch_bounds__(C::NT) step_fused2_tma_kernel(const Params P, const Coef<typename C::real> c,
+                                                                const StepPtrs S,
                                                                 const __grid_constant__ CUtensorMap tm_g,
                                                                 const __grid_constant__ CUtensorMap tm_u, int a_lo,
                                                                 int b_lo) {
@@ -1444,12 +1470,13 @@ __global__ void __launch_bounds__(C::NT) step_fused2_tma_kernel(const Params P, 
     if (threadIdx.x == 0 && S.err) atomicExch(S.err, 1);
     return;
   }
-  fused2_tile<C>(P, S, sg, su, sh, sn, x0, y0);
+  fused2_tile<C>(P, c, S, sg, su, sh, sn, x0, y0);
 }
 
 // frame tiles of a periodic lattice: the boxes gathered with wrapped loads
 template <class C>
-__global__ void __launch_bounds__(C::NT) step_fused2_edge_kernel(const Params P, const StepPtrs S, int ntx, int a_lo,
+__global__ void __launch_bounds__(C::NT) step_fused2_edge_kernel(const Params P, const Coef<typename C::real> c,
+                                                                 const StepPtrs S, int ntx, int a_lo,
                                                                  int a_hi, int b_lo, int b_hi) {
   using F = Fuse2Cfg<C>;
   using gs = typename C::gs;
@@ -1482,7 +1509,7 @@ __global__ void __launch_bounds__(C::NT) step_fused2_edge_kernel(const Params P,
     su[e] = u[(size_t)y * P.pitch + x];
   }
   __syncthreads();
-  fused2_tile<C>(P, S, sg, su, sh, sn, x0, y0);
+  fused2_tile<C>(P, c, S, sg, su, sh, sn, x0, y0);
 }
 
 // Fused iterations apply to lattices with every edge periodic and both sides
@@ -1501,9 +1528,10 @@ cudaError_t launch_step_fused2(const Params &P, const StepPtrs &S, cudaStream_t 
   const int nedge = ntx * nty - ni * nj;
   const bool beside = fork_begin(S, st, ni > 0 && nj > 0 && nedge > 0);
   cudaStream_t es = beside ? S.fork->side : st;
-  if (nedge > 0) step_fused2_edge_kernel<C><<<nedge, C::NT, F::SMEM, es>>>(P, S, ntx, a_lo, a_hi, b_lo, b_hi);
+  const auto c = make_coef<typename C::gs, typename C::real>(P);
+  if (nedge > 0) step_fused2_edge_kernel<C><<<nedge, C::NT, F::SMEM, es>>>(P, c, S, ntx, a_lo, a_hi, b_lo, b_hi);
   if (ni > 0 && nj > 0)
-    step_fused2_tma_kernel<C><<<dim3(ni, nj), C::NT, F::SMEM, st>>>(P, S, *(const CUtensorMap *)S.tm_g,
+    step_fused2_tma_kernel<C><<<dim3(ni, nj), C::NT, F::SMEM, st>>>(P, c, S, *(const CUtensorMap *)S.tm_g,
                                                                       *(const CUtensorMap *)S.tm_u, a_lo, b_lo);
   fork_end(S, st, beside);
   return cudaGetLastError();
@@ -1604,7 +1632,8 @@ __device__ __forceinline__ bool march_wait(uint64_t *bar, uint32_t parity) {
 }
 
 template <class C, class M>
-__global__ void __launch_bounds__(M::NT) step_march_kernel(const Params P, const StepPtrs S,
+__global__ void __launch_bounds__(M::NT) step_march_kernel(const Params P, const Coef<typename C::real> k,
+                                                           const StepPtrs S,
                                                            const __grid_constant__ CUtensorMap tm_g,
                                                            const __grid_constant__ CUtensorMap tm_u, int a_lo, int ni,
                                                            int y_first, int y_last) {
@@ -1636,11 +1665,8 @@ __global__ void __launch_bounds__(M::NT) step_march_kernel(const Params P, const
     march_issue<M>(dsm, &bar[j % D], tm_g, tm_u, x0, y + 3, RB, gbase, y + 2, RB, ubase);
   };
 
-  const R inv = gscale_inv<gs, R>(P), scl = gscale<gs, R>(P);
-  const R kap = (R)P.kappa * inv, hdx = R(0.5) * (R)P.inv_dx;
-  const R lam = (R)P.lam, mu = (R)P.mu;
-  const CollideK<R> K = collide_k<R>((R)P.omega, (R)P.sigma, scl);
-  const R sbx = (R)(P.rho0 * P.body[0]), sby = (R)(P.rho0 * P.body[1]);
+  const R kap = k.kap, hdx = k.hdx, scl = k.scl, lam = k.lam, mu = k.mu, sbx = k.sbx, sby = k.sby;
+  const CollideK<R> &K = k.K;
   const size_t plane = (size_t)P.ny * P.pitch;
   gs *__restrict__ go = (gs *)S.g_out;
   us *__restrict__ uo = (us *)S.u_out;
@@ -1755,7 +1781,8 @@ cudaError_t launch_step_march(const Params &P, const StepPtrs &S, cudaStream_t s
   if (ni > 0 && nj > 0) {
     const int y_first = b_lo * C::TY, y_last = b_hi * C::TY;
     const int nseg = (y_last - y_first + M::SH - 1) / M::SH;
-    step_march_kernel<C, M><<<ni * nseg, M::NT, M::SMEM, st>>>(P, S, *(const CUtensorMap *)S.tm_g,
+    step_march_kernel<C, M><<<ni * nseg, M::NT, M::SMEM, st>>>(P, make_coef<typename C::gs, typename C::real>(P), S,
+                                                               *(const CUtensorMap *)S.tm_g,
                                                                *(const CUtensorMap *)S.tm_u, a_lo, ni, y_first, y_last);
   }
   if (!beside) launch_edge<C>(P, S, nedge, ntx, a_lo, a_hi, b_lo, b_hi, st);
@@ -1862,23 +1889,23 @@ __device__ void load_r2_from_state(typename C::Smem &sm, const Params &P, const 
 // Alg. 1 "Initialise": r0 = -rho0 tr H0, Pi0 = Pi(H0), f0 = feq(r0, rho0 v0 - dt/2 S0, Pi0),
 // then the first collision (with S0) gives the stored g.
 template <class C>
-__global__ void __launch_bounds__(C::NT) init_kernel(const Params P, typename C::gs *g, typename C::us *u,
+__global__ void __launch_bounds__(C::NT) init_kernel(const Params P, const Coef<typename C::real> c, typename C::gs *g, typename C::us *u,
                                                      typename C::real *bnd, const double *u0, const double *v0) {
   using R = typename C::real;
   __shared__ typename C::Smem sm;
   const int x0 = blockIdx.x * C::TX, y0 = blockIdx.y * C::TY;
   load_r2_from_double<C>(sm, P, u0, x0, y0);
   __syncthreads();
-  phase_n<C, true, true>(sm, P, x0, y0, bnd);
+  phase_n<C, true, true>(sm, P, c, x0, y0, bnd);
   __syncthreads();
   const size_t plane = (size_t)P.ny * P.pitch;
-  const R idx_ = (R)P.inv_dx, scl = gscale<typename C::gs, R>(P);
+  const R idx_ = c.idx, scl = c.scl;
   const int tx = threadIdx.x % C::TX, ty = threadIdx.x / C::TX;
   for (int i = 0; i < C::CPT; ++i) {
     const int lx = tx, ly = ty + i * C::NTY, x = x0 + lx, y = y0 + ly;
     if (x >= P.nx || y >= P.ny) continue;
     R Sx, Sy, H[4];
-    Fd<C, true>::div(sm, P, lx + 1, ly + 1, x, y, idx_, (R)(P.rho0 * P.body[0]), (R)(P.rho0 * P.body[1]), Sx, Sy);
+    Fd<C, true>::div(sm, P, lx + 1, ly + 1, x, y, idx_, c.sbx, c.sby, Sx, Sy);
     Fd<C, true>::grad(sm, P, lx + 1, ly + 1, x, y, idx_, H);
     const size_t i0 = (size_t)y * P.nx + x;
     const R trH = H[0] + H[3];
@@ -1897,7 +1924,7 @@ __global__ void __launch_bounds__(C::NT) init_kernel(const Params P, typename C:
       const R eAe = R(ex(q) * ex(q)) * Axx + R(2 * ex(q) * ey(q)) * Axy + R(ey(q) * ey(q)) * Ayy;
       f[q] = wq<R>(q) * (rq + R(ex(q)) * jx + R(ey(q)) * jy + R(1.5) * eAe - R(0.5) * (Axx + Ayy)) * scl;
     }
-    collide<R>(f, Sx, Sy, collide_k<R>((R)P.omega, (R)P.sigma, scl));
+    collide<R>(f, Sx, Sy, c.K);
     const size_t idx = (size_t)y * P.pitch + x;
     for (int q = 0; q < 9; ++q) gstore(g, q * plane + idx, f[q], scl);
     u[idx] = sm.u[ly + 2][lx + 2];
@@ -1910,11 +1937,12 @@ __global__ void __launch_bounds__(C::NT) init_kernel(const Params P, typename C:
 // hr = dt / (2 rho0) are formed once per thread by the caller, so that no
 // node divides in FP64.
 template <class C>
-__device__ __forceinline__ void node_fields(const typename C::Smem &sm, const Params &P, const typename C::gs *g,
+__device__ __forceinline__ void node_fields(const typename C::Smem &sm, const Params &P,
+                                            const Coef<typename C::real> &c, const typename C::gs *g,
                                             size_t plane, size_t idx, int lx, int ly, int x, int y, size_t o,
                                             double cr, double hr, double *uo, double *vo, double *Po) {
   using R = typename C::real;
-  const R idx_ = (R)P.inv_dx;
+  const R idx_ = c.idx;
   if (uo) {
     const double2 uv = u_value(sm.u[ly + 2][lx + 2]);
     uo[2 * o] = uv.x;
@@ -1922,9 +1950,9 @@ __device__ __forceinline__ void node_fields(const typename C::Smem &sm, const Pa
   }
   if (vo) {
     R Sx, Sy;
-    Fd<C, true>::div(sm, P, lx + 1, ly + 1, x, y, idx_, (R)(P.rho0 * P.body[0]), (R)(P.rho0 * P.body[1]), Sx, Sy);
+    Fd<C, true>::div(sm, P, lx + 1, ly + 1, x, y, idx_, c.sbx, c.sby, Sx, Sy);
     // g is held in units of g * 2^gshift (1 unless FP16 storage)
-    const R inv = gscale_inv<typename C::gs, R>(P);
+    const R inv = c.inv;
     R gq[9], m1x, m1y;
     for (int q = 1; q < 9; ++q) gq[q] = gload(g, q * plane + idx, inv);
     first_moment(gq, m1x, m1y);
@@ -1932,7 +1960,7 @@ __device__ __forceinline__ void node_fields(const typename C::Smem &sm, const Pa
     vo[2 * o + 1] = fma(cr, (double)(m1y * inv), -(hr * (double)Sy));
   }
   if (Po) {
-    const R mu = (R)P.mu;
+    const R mu = c.mu;
     R H[4];
     Fd<C, true>::grad(sm, P, lx + 1, ly + 1, x, y, idx_, H);
     const R trH = H[0] + H[3];
@@ -1946,7 +1974,8 @@ __device__ __forceinline__ void node_fields(const typename C::Smem &sm, const Pa
 // u, v and P at every node (x fastest); N on the tile + 1 only when v or P is
 // asked for
 template <class C>
-__global__ void __launch_bounds__(C::NT) fields_kernel(const Params P, const typename C::gs *g, const typename C::us *u,
+__global__ void __launch_bounds__(C::NT) fields_kernel(const Params P, const Coef<typename C::real> c,
+                                                       const typename C::gs *g, const typename C::us *u,
                                                        double *uo, double *vo, double *Po) {
   using R = typename C::real;
   __shared__ typename C::Smem sm;
@@ -1954,7 +1983,7 @@ __global__ void __launch_bounds__(C::NT) fields_kernel(const Params P, const typ
   load_r2_from_state<C>(sm, P, u, x0, y0);
   __syncthreads();
   if (vo || Po) {
-    phase_n<C, true>(sm, P, x0, y0, (R *)nullptr);
+    phase_n<C, true>(sm, P, c, x0, y0, (R *)nullptr);
     __syncthreads();
   }
   const size_t plane = (size_t)P.ny * P.pitch;
@@ -1963,7 +1992,7 @@ __global__ void __launch_bounds__(C::NT) fields_kernel(const Params P, const typ
   for (int i = 0; i < C::CPT; ++i) {
     const int lx = tx, ly = ty + i * C::NTY, x = x0 + lx, y = y0 + ly;
     if (x >= P.nx || y >= P.ny) continue;
-    node_fields<C>(sm, P, g, plane, (size_t)y * P.pitch + x, lx, ly, x, y, (size_t)y * P.nx + x, cr, hr, uo, vo,
+    node_fields<C>(sm, P, c, g, plane, (size_t)y * P.pitch + x, lx, ly, x, y, (size_t)y * P.nx + x, cr, hr, uo, vo,
                    Po);
   }
 }
@@ -2134,7 +2163,7 @@ __global__ void probe_kernel(const Params P, const typename C::us *u, const int3
 template <class C>
 cudaError_t launch_init(const Params &P, void *g, void *u, void *b, const double *u0, const double *v0, cudaStream_t st) {
   dim3 grid((P.nx + C::TX - 1) / C::TX, (P.ny + C::TY - 1) / C::TY);
-  init_kernel<C><<<grid, C::NT, 0, st>>>(P, (typename C::gs *)g, (typename C::us *)u, (typename C::real *)b, u0, v0);
+  init_kernel<C><<<grid, C::NT, 0, st>>>(P, make_coef<typename C::gs, typename C::real>(P), (typename C::gs *)g, (typename C::us *)u, (typename C::real *)b, u0, v0);
   return cudaGetLastError();
 }
 
@@ -2142,7 +2171,7 @@ template <class C>
 cudaError_t launch_fields(const Params &P, const void *g, const void *u, double *uo, double *vo, double *Po,
                           cudaStream_t st) {
   dim3 grid((P.nx + C::TX - 1) / C::TX, (P.ny + C::TY - 1) / C::TY);
-  fields_kernel<C><<<grid, C::NT, 0, st>>>(P, (const typename C::gs *)g, (const typename C::us *)u, uo, vo, Po);
+  fields_kernel<C><<<grid, C::NT, 0, st>>>(P, make_coef<typename C::gs, typename C::real>(P), (const typename C::gs *)g, (const typename C::us *)u, uo, vo, Po);
   return cudaGetLastError();
 }
 

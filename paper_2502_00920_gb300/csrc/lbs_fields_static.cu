@@ -56,7 +56,8 @@ unsigned long long current_context_id() {
 
 // u, v, P of rows [y_lo, y_hi) into dense row-block arrays (x fastest)
 template <class C>
-__global__ void __launch_bounds__(C::NT) fields_rows_kernel(const Params P, const typename C::gs *g,
+__global__ void __launch_bounds__(C::NT) fields_rows_kernel(const Params P, const Coef<typename C::real> c,
+                                                            const typename C::gs *g,
                                                             const typename C::us *u, int y_lo, int y_hi, double *uo,
                                                             double *vo, double *Po) {
   using R = typename C::real;
@@ -65,7 +66,7 @@ __global__ void __launch_bounds__(C::NT) fields_rows_kernel(const Params P, cons
   load_r2_from_state<C>(sm, P, u, x0, y0);
   __syncthreads();
   if (vo || Po) {
-    phase_n<C, true>(sm, P, x0, y0, (R *)nullptr);
+    phase_n<C, true>(sm, P, c, x0, y0, (R *)nullptr);
     __syncthreads();
   }
   const size_t plane = (size_t)P.ny * P.pitch;
@@ -74,7 +75,7 @@ __global__ void __launch_bounds__(C::NT) fields_rows_kernel(const Params P, cons
   for (int i = 0; i < C::CPT; ++i) {
     const int lx = tx, ly = ty + i * C::NTY, x = x0 + lx, y = y0 + ly;
     if (x >= P.nx || y < y_lo || y >= y_hi) continue;
-    node_fields<C>(sm, P, g, plane, (size_t)y * P.pitch + x, lx, ly, x, y, (size_t)(y - y_lo) * P.nx + x, cr, hr,
+    node_fields<C>(sm, P, c, g, plane, (size_t)y * P.pitch + x, lx, ly, x, y, (size_t)(y - y_lo) * P.nx + x, cr, hr,
                    uo, vo, Po);
   }
 }
@@ -85,7 +86,8 @@ cudaError_t launch_rows(const Params &P, const void *g, const void *u, int y_lo,
   using C = Cfg<Pr, 32, 16, 8>;
   const int b_first = y_lo / C::TY, b_last = (y_hi - 1) / C::TY;
   dim3 grid((P.nx + C::TX - 1) / C::TX, b_last - b_first + 1);
-  fields_rows_kernel<C><<<grid, C::NT, 0, st>>>(P, (const typename C::gs *)g, (const typename C::us *)u, y_lo, y_hi,
+  fields_rows_kernel<C><<<grid, C::NT, 0, st>>>(P, make_coef<typename C::gs, typename C::real>(P),
+                                                (const typename C::gs *)g, (const typename C::us *)u, y_lo, y_hi,
                                                 uo, vo, Po);
   return cudaGetLastError();
 }

@@ -79,6 +79,7 @@ struct TileShape {
 // buffers of each state array, and its iteration counter and end.
 struct BatchLattice {
   Params P;
+  double coef[32];  // Coef<real> of the batch's precision (Launchers::coef)
   void *g[2], *u[2], *b[2];
   int64_t k;     // iteration at the start of the current chunk (launch `it` of the
                  // chunk steps iteration k + it, buffers [(k + it) & 1]); advanced
@@ -118,6 +119,9 @@ struct Launchers {
   // last iteration of an odd count under a fused variant); one or two kernels
   cudaError_t (*step1)(const Params &p, const StepPtrs &s, cudaStream_t st);
   int (*kernels_per_step1)(const Params &p);
+  // the scheme's coefficients in the precision's compute type (Coef<real>) for
+  // a batch's table (out: 32 doubles of room)
+  void (*coef)(const Params &p, void *out);
   // n iterations in one cooperative launch, for the lattices where that is
   // faster than launching every iteration (resident_applies)
   bool (*resident_applies)(const Params &p);

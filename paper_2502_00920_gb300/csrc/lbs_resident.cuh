@@ -46,17 +46,6 @@ __device__ __forceinline__ bool grid_barrier(unsigned *count, unsigned target, i
   return __syncthreads_and(ok) != 0;
 }
 
-// keep a loop-invariant value in its register (the compiler otherwise
-// converts the double parameter again in every iteration)
-__device__ __forceinline__ float pinned(float v) {
-  asm volatile("" : "+f"(v));
-  return v;
-}
-__device__ __forceinline__ double pinned(double v) {
-  asm volatile("" : "+d"(v));
-  return v;
-}
-
 // The own-value wall rules of wall_rules() for one node with what does not
 // change between iterations taken out: sev holds the edges' values in the
 // compute type, js the momentum of a diagonal link between two Dirichlet walls
@@ -121,8 +110,9 @@ constexpr int kSevBatch = 32;
 // barrier's counters are zero between launches: the last block to leave clears
 // them.  A launch that finds the error flag set does nothing.
 template <class C, bool LIN>
-__global__ void __launch_bounds__(C::NT) resident_kernel(const Params P, const ResidentPtrs S, int parity, int64_t k0,
-                                                         int n, int ntx) {
+__global__ void __launch_bounds__(C::NT) resident_kernel(const Params P, const Coef<typename C::real> c,
+                                                         const ResidentPtrs S, int parity, int64_t k0, int n,
+                                                         int ntx) {
   using gs = typename C::gs;
   using us = typename C::us;
   using R = typename C::real;
@@ -138,12 +128,7 @@ __global__ void __launch_bounds__(C::NT) resident_kernel(const Params P, const R
   const int x0 = (int)(blockIdx.x % ntx) * C::TX, y0 = (int)(blockIdx.x / ntx) * C::TY;
   const int plane = P.ny * P.pitch;
   const bool walls = !(P.per_x && P.per_y);
-  const R inv = pinned(gscale_inv<gs, R>(P)), scl = pinned(gscale<gs, R>(P));
-  const R kap = pinned((R)P.kappa * inv), idx_ = pinned((R)P.inv_dx);
-  const R lam = pinned((R)P.lam), mu = pinned((R)P.mu);
-  const CollideK<R> K = collide_k<R>(pinned((R)P.omega), pinned((R)P.sigma), scl);
-  const R sbx = pinned((R)(P.rho0 * P.body[0])), sby = pinned((R)(P.rho0 * P.body[1]));
-  const R ics2 = pinned((R)P.inv_cs2 * scl), cj = pinned((R)(P.c * P.inv_cs2) * scl);
+  const R scl = c.scl, kap = c.kap, idx_ = c.idx, sbx = c.sbx, sby = c.sby, ics2 = c.ics2, cj = c.cj;
 
   // phase 1: this thread's node of R2
   const int e = threadIdx.x;
@@ -275,7 +260,7 @@ __global__ void __launch_bounds__(C::NT) resident_kernel(const Params P, const R
         if constexpr (LIN) {
           R wnl[4];
           wall_n<true>(P, bnd, xw, yw, x, y, wnl);
-          wall_rules<R, gs, true, true>(P, bnd, g, ev, x, y, xw, yw, wnl, g0, mask, f, scl);
+          wall_rules<R, gs, true, true>(P, bnd, g, ev, x, y, xw, yw, wnl, g0, mask, f, ics2, cj);
         } else {
           wall_rules_own<R>(mask, crossx, crossy, dirx, diry, sgx, sgy, ics2, cj, wn, ev[xw < 0 ? 0 : xw],
                             ev[yw < 0 ? 0 : yw], ev[corner], g0, f);
@@ -296,7 +281,7 @@ __global__ void __launch_bounds__(C::NT) resident_kernel(const Params P, const R
       H[1] = dyx * sy1;
       H[2] = dxy * sx1;
       H[3] = dyy * sy1;
-      material<R>(P, lam, mu, H, N);
+      material<R>(P, c.lam, c.mu, H, N);
 #pragma unroll
       for (int m = 0; m < 4; ++m) sn[m][e] = N[m];
       if (keep1) {
@@ -309,7 +294,7 @@ __global__ void __launch_bounds__(C::NT) resident_kernel(const Params P, const R
     if (own) {
       const R Sx = fmr(sn[0][nx1] - sn[0][nx0], sx2, fmr(sn[1][ny1] - sn[1][ny0], sy2, sbx));
       const R Sy = fmr(sn[2][nx1] - sn[2][nx0], sx2, fmr(sn[3][ny1] - sn[3][ny0], sy2, sby));
-      collide<R>(f, Sx, Sy, K);
+      collide<R>(f, Sx, Sy, c.K);
       gs *go = (gs *)S.g[p ^ 1];
 #pragma unroll
       for (int q = 0; q < 9; ++q) {
@@ -380,7 +365,8 @@ int resident_shape(const Params &P, int large_most) {
 template <class C>
 cudaError_t launch_resident_c(const Params &P, const ResidentPtrs &S, int parity, int64_t k0, int n, cudaStream_t st) {
   int ntx = (P.nx + C::TX - 1) / C::TX, nty = (P.ny + C::TY - 1) / C::TY;
-  void *args[] = {(void *)&P, (void *)&S, &parity, &k0, &n, &ntx};
+  auto c = make_coef<typename C::gs, typename C::real>(P);
+  void *args[] = {(void *)&P, &c, (void *)&S, &parity, &k0, &n, &ntx};
   const void *kernel = P.extrap ? (const void *)resident_kernel<C, true> : (const void *)resident_kernel<C, false>;
   return cudaLaunchCooperativeKernel(kernel, dim3(ntx * nty), dim3(C::NT), args, 0, st);
 }

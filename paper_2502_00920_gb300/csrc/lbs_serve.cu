@@ -471,6 +471,7 @@ void run(lbs_server *s) {
         lbs_handle *h = res[i]->h;
         BatchLattice &B = hl[i];
         B.P = h->P;
+        L.coef(h->P, B.coef);
         for (int p = 0; p < 2; ++p) {
           B.g[p] = h->g[p];
           B.u[p] = h->u[p];
