@@ -458,17 +458,18 @@ __device__ void wall_rules(const Params &P, const R *bnd, const G *g, const doub
 // each less the dt/2 S part of j, which combines with the forcing term
 // (1 - 1/(2 tau)) psi dt into w_q sigma e_q.S per population (sigma = c dt / cs^2;
 // its first moment is sigma S / 3 = dt S / c, the momentum the source adds).
+// The four odd parts have only two degrees of freedom beside the momentum:
+// with tx = 6 ox and ty = 6 oy, 12 o57 = -(tx + ty) and 12 o68 = tx - ty.
 // So g_q = f_q - omega (f - feq)_q + w_q sigma e_q.S.  The same algebra as
 // the literal moment form, but every intermediate is of the size of the
 // populations, so single-precision rounding stays at the level of the stored
 // values instead of that of the second moments.
-// Per-thread constants of the collision: -omega, the relaxation of the even
-// part per unit Q for the axis (omega/18) and diagonal (-omega/36)
-// populations, and the forcing weights sigma/9 and sigma/36 times the storage
-// scale of g (the source arrives unscaled).
+// Constants of the collision: -omega, the relaxation of the even part per unit
+// Q for the axis (omega/18) and diagonal (-omega/36) populations, and the
+// forcing weights sigma/9 and sigma/36 times the storage scale of g.
 template <class R>
 struct CollideK {
-  R mo, m6, m9, m12, a1, a5, s9, s36;
+  R mo, m6, m9, p3, a1, a5, s9, s36;
 };
 template <class R>
 __host__ __device__ __forceinline__ CollideK<R> collide_k(R omega, R sigma, R scl) {
@@ -476,7 +477,7 @@ __host__ __device__ __forceinline__ CollideK<R> collide_k(R omega, R sigma, R sc
   return {-omega,
           -omega * (R(1) / R(6)),
           -omega * (R(1) / R(9)),
-          -omega * (R(1) / R(12)),
+          omega * (R(1) / R(3)),
           omega * (R(1) / R(18)),
           -omega * (R(1) / R(36)),
           ss * (R(1) / R(9)),
@@ -485,29 +486,37 @@ __host__ __device__ __forceinline__ CollideK<R> collide_k(R omega, R sigma, R sc
 
 // Each opposite pair takes the even relaxation A = Q a1 or Q a5 (the same for
 // both) and the odd part b = -omega o + forcing with opposite signs:
-// g = (f + A) +- b; in FP64 the product Q a is fused into the population's
-// own add, g = fma(Q, a, f) +- b.
+// g = (f + A) +- b.  In FP64, where the pipe's slots set the time, the product
+// Q a is fused into the population's own add, the source arrives times sigma/9
+// (Coef's idxs, sbxs), and the diagonal pairs take their b from
+//   4 b57 = Cx + Cy, 4 b68 = Cy - Cx with Cx = (omega/3) tx + (sigma/9) Sx
+// (-omega o57 = omega (tx + ty) / 12): 39 slots a node where forming t57, t68
+// and their forcing apart took 47.
 template <class R>
 __device__ __forceinline__ void collide(R f[9], R Sx, R Sy, const CollideK<R> &K) {
   const R s13 = f[1] + f[3], s24 = f[2] + f[4], s57 = f[5] + f[7], s68 = f[6] + f[8];
   const R d13 = f[1] - f[3], d24 = f[2] - f[4], d57 = f[5] - f[7], d68 = f[6] - f[8];
   // (the products by 2 and 4 are exact)
   const R Q = fmr(R(4), s57 + s68, fmr(R(-2), s13 + s24, f[0]));
-  const R fx = Sx * K.s9, fy = Sy * K.s9;
-  const R f57 = (Sx + Sy) * K.s36, f68 = (Sy - Sx) * K.s36;
-  const R A1 = Q * K.a1, A5 = Q * K.a5;  // (single precision; unused in FP64)
-  R bx, by, b57, b68;
   if constexpr (sizeof(R) == 8) {
-    // the odd parts, ox = (d13 - 2 (d57 - d68)) / 6 and so on, enter only as
-    // -omega times them: the division goes into that factor (the products by
-    // 2 and 4 are exact), four FP64 operations fewer per node
+    // (the products by 2 and 1/4 are exact)
     const R tx = fmr(R(-2), d57 - d68, d13), ty = fmr(R(-2), d57 + d68, d24);
-    const R t57 = fmr(R(4), d57, -(d13 + d24)), t68 = fmr(R(4), d68, -(d24 - d13));
-    bx = fmr(tx, K.m6, fx);
-    by = fmr(ty, K.m6, fy);
-    b57 = fmr(t57, K.m12, f57);
-    b68 = fmr(t68, K.m12, f68);
+    const R bx = fmr(tx, K.m6, Sx), by = fmr(ty, K.m6, Sy);
+    const R cx = fmr(tx, K.p3, Sx), cy = fmr(ty, K.p3, Sy);
+    const R b57 = cx + cy, b68 = cy - cx;
+    f[0] = fmr(Q, K.m9, f[0]);
+    f[1] = fmr(Q, K.a1, f[1]) + bx;
+    f[3] = fmr(Q, K.a1, f[3]) - bx;
+    f[2] = fmr(Q, K.a1, f[2]) + by;
+    f[4] = fmr(Q, K.a1, f[4]) - by;
+    f[5] = fmr(R(0.25), b57, fmr(Q, K.a5, f[5]));
+    f[7] = fmr(R(-0.25), b57, fmr(Q, K.a5, f[7]));
+    f[6] = fmr(R(0.25), b68, fmr(Q, K.a5, f[6]));
+    f[8] = fmr(R(-0.25), b68, fmr(Q, K.a5, f[8]));
   } else {
+    const R fx = Sx * K.s9, fy = Sy * K.s9;
+    const R f57 = (Sx + Sy) * K.s36, f68 = (Sy - Sx) * K.s36;
+    const R A1 = Q * K.a1, A5 = Q * K.a5;
     // (single precision keeps the odd parts themselves: the form above
     // measured slower for FP16 storage, whose kernel is issue-bound)
     const R c3 = R(1) / R(3), c6 = R(1) / R(6), c12 = R(1) / R(12);
@@ -515,23 +524,8 @@ __device__ __forceinline__ void collide(R f[9], R Sx, R Sy, const CollideK<R> &K
     const R oy = fmr(d24, c6, -((d57 + d68) * c3));
     const R o57 = fmr(d57, c3, -((d13 + d24) * c12));
     const R o68 = fmr(d68, c3, -((d24 - d13) * c12));
-    bx = fmr(K.mo, ox, fx);
-    by = fmr(K.mo, oy, fy);
-    b57 = fmr(K.mo, o57, f57);
-    b68 = fmr(K.mo, o68, f68);
-  }
-  if constexpr (sizeof(R) == 8) {
-    // three FP64 multiplies fewer per node
-    f[0] = fmr(Q, K.m9, f[0]);
-    f[1] = fmr(Q, K.a1, f[1]) + bx;
-    f[3] = fmr(Q, K.a1, f[3]) - bx;
-    f[2] = fmr(Q, K.a1, f[2]) + by;
-    f[4] = fmr(Q, K.a1, f[4]) - by;
-    f[5] = fmr(Q, K.a5, f[5]) + b57;
-    f[7] = fmr(Q, K.a5, f[7]) - b57;
-    f[6] = fmr(Q, K.a5, f[6]) + b68;
-    f[8] = fmr(Q, K.a5, f[8]) - b68;
-  } else {
+    const R bx = fmr(K.mo, ox, fx), by = fmr(K.mo, oy, fy);
+    const R b57 = fmr(K.mo, o57, f57), b68 = fmr(K.mo, o68, f68);
     // (single precision keeps the separate products: the fused form takes
     // the FP16-storage TMA kernel past 64 registers)
     f[0] = fmr(K.mo, Q * (R(1) / R(9)), f[0]);
@@ -558,6 +552,9 @@ struct Coef {
   R lam, mu;
   R idx, hdx;    // 1 / dx, 1 / (2 dx)
   R sbx, sby;    // rho0 b
+  // the same as the collision takes the source: times sigma/9 in FP64
+  R idxs, hdxs, sbxs, sbys;
+  R h2, c1;      // hdx^2, lam / (2 mu) (FP64 neo-Hooke)
   R ics2, cj;    // 1 / cs^2 and c / cs^2 in storage units of g (wall rules)
   CollideK<R> K;
 };
@@ -576,7 +573,55 @@ __host__ __device__ inline Coef<R> make_coef(const Params &P) {
   k.ics2 = (R)P.inv_cs2 * k.scl;
   k.cj = (R)(P.c * P.inv_cs2) * k.scl;
   k.K = collide_k<R>((R)P.omega, (R)P.sigma, k.scl);
+  const R src = sizeof(R) == 8 ? k.K.s9 : R(1);
+  k.idxs = k.idx * src;
+  k.hdxs = R(0.5) * k.idxs;
+  k.sbxs = k.sbx * src;
+  k.sbys = k.sby * src;
+  k.h2 = k.hdx * k.hdx;
+  k.c1 = R(0.5) * k.lam / k.mu;
   return k;
+}
+
+// N of a node from the differences of u over two spacings (dxx = the
+// difference of u_x along x, and so on; on a wall node of the axis, onex /
+// oney, the one-sided difference over one spacing).  In FP64 neo-Hooke takes
+// the differences themselves, with H = hdx D folded into its coefficients (a
+// one-sided difference is doubled first, exactly); otherwise H is formed and
+// handed to material().
+template <class R>
+__device__ __forceinline__ void stress_n(const Params &P, const Coef<R> &c, R dxx, R dxy, R dyx, R dyy, bool onex,
+                                         bool oney, R N[4]) {
+  if constexpr (sizeof(R) == 8) {
+    if (P.model == LBS_NH) {
+      if (onex) {
+        dxx += dxx;
+        dxy += dxy;
+      }
+      if (oney) {
+        dyx += dyx;
+        dyy += dyy;
+      }
+      // a = J - 1 = tr H + det H; with m = mu / J, q = m (2 + a) and
+      // l = lam a (a + 2) / (2 J) = c1 a q:
+      //   N11 = (l + m a - q tr H) + l H22 - m a H11,  N12 = -(m a + l) H21
+      const R trH = c.hdx * (dxx + dyy);
+      const R a = fmr(c.h2, fmr(dxx, dyy, -(dyx * dxy)), trH);
+      const R m = c.mu * (R(1) / (R(1) + a));
+      const R ma = m * a, q = m * (R(2) + a);
+      const R l = (c.c1 * a) * q;
+      const R d = l + fmr(-q, trH, ma);
+      const R mah = c.hdx * ma, lh = c.hdx * l, s = mah + lh;
+      N[0] = fmr(-mah, dxx, fmr(lh, dyy, d));
+      N[1] = -(s * dxy);
+      N[2] = -(s * dyx);
+      N[3] = fmr(-mah, dyy, fmr(lh, dxx, d));
+      return;
+    }
+  }
+  const R sx = onex ? c.idx : c.hdx, sy = oney ? c.idx : c.hdx;
+  const R H[4] = {dxx * sx, dyx * sy, dxy * sx, dyy * sy};
+  material<R>(P, c.lam, c.mu, H, N);
 }
 
 // ------------------------------------------------------------------ tiles
@@ -722,6 +767,18 @@ struct Fd {
     H[2] = dxy * sx;
     H[3] = dyy * sy;
   }
+  // N at R1 position (rx, ry) from su
+  static __device__ __forceinline__ void stress(const typename C::Smem &sm, const Params &P, const Coef<R> &c, int rx,
+                                                int ry, int gxn, int gyn, R N[4]) {
+    R dxx, dxy, dyx, dyy;
+    const int cx = rx + 1, cy = ry + 1;
+    int xa, xb, ya, yb;
+    bool onex, oney;
+    fd_taps<EDGE>(P, cx, cy, gxn, gyn, xa, xb, ya, yb, onex, oney);
+    udiff(sm.u[cy][xa], sm.u[cy][xb], dxx, dxy);
+    udiff(sm.u[ya][cx], sm.u[yb][cx], dyx, dyy);
+    stress_n<R>(P, c, dxx, dxy, dyx, dyy, onex, oney, N);
+  }
   // S = div N + (sbx, sby) at R1 position (rx, ry) of a tile node
   static __device__ __forceinline__ void div(const typename C::Smem &sm, const Params &P, int rx, int ry, int gxn,
                                              int gyn, R idx_, R sbx, R sby, R &Sx, R &Sy) {
@@ -745,9 +802,8 @@ __device__ __forceinline__ void phase_n(typename C::Smem &sm, const Params &P, c
     const int rx = e % C::R1W, ry = e / C::R1W;
     int gx = x0 - 1 + rx, gy = y0 - 1 + ry;
     if (EDGE && !locate(P, gx, gy)) continue;
-    R H[4], N[4];
-    Fd<C, EDGE>::grad(sm, P, rx, ry, gx, gy, k.idx, H);
-    material<R>(P, k.lam, k.mu, H, N);
+    R N[4];
+    Fd<C, EDGE>::stress(sm, P, k, rx, ry, gx, gy, N);
 #pragma unroll
     for (int m = 0; m < 4; ++m) sm.n[m][ry][rx] = N[m];
     if (EDGE && bnd_out && r1_own_node<C>(P, x0, y0, rx, ry)) {
@@ -824,7 +880,7 @@ __device__ __forceinline__ void step_tile(const Params &P, const Coef<typename C
     const int x = x0 + lx, y = y0 + ly;
     if (EDGE && (x >= P.nx || y >= P.ny)) continue;
     R Sx, Sy;
-    Fd<C, EDGE>::div(sm, P, lx + 1, ly + 1, x, y, c.idx, c.sbx, c.sby, Sx, Sy);
+    Fd<C, EDGE>::div(sm, P, lx + 1, ly + 1, x, y, c.idxs, c.sbxs, c.sbys, Sx, Sy);
     collide<R>(f[i], Sx, Sy, c.K);
     const size_t idx = (size_t)y * P.pitch + x;
 #pragma unroll
@@ -1057,7 +1113,6 @@ __device__ __forceinline__ void tma_tile(const Params &P, const Coef<typename C:
   // phase 2: N on R1
   constexpr int W1 = C::TX + 2, H1 = C::TY + 2, NE = W1 * H1, NPER = (NE + C::NT - 1) / C::NT;
   const int tx = threadIdx.x % C::TX, ty = threadIdx.x / C::TX;
-  const R hdx = c.hdx;
   // own nodes' u(t+dt), read before N may overwrite the box
   us uown[C::CPT];
 #pragma unroll
@@ -1070,14 +1125,10 @@ __device__ __forceinline__ void tma_tile(const Params &P, const Coef<typename C:
       if (e >= NE) break;
       const int rx = e % W1, ry = e / W1;
       const int at = (ry + 1) * T::UW + (rx + 1);
-      R dxx, dxy, dyx, dyy, H[4], N[4];
+      R dxx, dxy, dyx, dyy, N[4];
       udiff(su[at + 1], su[at - 1], dxx, dxy);
       udiff(su[at + T::UW], su[at - T::UW], dyx, dyy);
-      H[0] = dxx * hdx;
-      H[1] = dyx * hdx;
-      H[2] = dxy * hdx;
-      H[3] = dyy * hdx;
-      material<R>(P, c.lam, c.mu, H, N);
+      stress_n<R>(P, c, dxx, dxy, dyx, dyy, false, false, N);
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
         if constexpr (T::N_IN_U) nreg[k][m] = N[m];
@@ -1099,7 +1150,7 @@ __device__ __forceinline__ void tma_tile(const Params &P, const Coef<typename C:
   __syncthreads();
   // phase 3: stream again from shared memory, source, collision, store
   const size_t plane = (size_t)P.ny * P.pitch;
-  const R sbx = c.sbx, sby = c.sby;
+  const R hdx = c.hdxs, sbx = c.sbxs, sby = c.sbys;
   gs *__restrict__ go = (gs *)S.g_out;
   us *__restrict__ uo = (us *)S.u_out;
 #pragma unroll
@@ -1359,7 +1410,7 @@ __device__ __forceinline__ void fused2_tile(const Params &P, const Coef<typename
   using R = typename C::real;
   using us = typename C::us;
   using gs = typename C::gs;
-  const R hdx = c.hdx, sbx = c.sbx, sby = c.sby;
+  const R hdx = c.hdxs, sbx = c.sbxs, sby = c.sbys;
   // u(t+dt) at node offset (i, j) from the populations of array A (g box or g1)
   auto advance_u = [&](auto A, int i, int j) {
     R p[9], o[9];
@@ -1376,14 +1427,10 @@ __device__ __forceinline__ void fused2_tile(const Params &P, const Coef<typename
   };
   // N at node offset (i, j) from u in the u box
   auto stress = [&](int i, int j) {
-    R dxx, dxy, dyx, dyy, H[4], N[4];
+    R dxx, dxy, dyx, dyy, N[4];
     udiff(su[F::u(i + 1, j)], su[F::u(i - 1, j)], dxx, dxy);
     udiff(su[F::u(i, j + 1)], su[F::u(i, j - 1)], dyx, dyy);
-    H[0] = dxx * hdx;
-    H[1] = dyx * hdx;
-    H[2] = dxy * hdx;
-    H[3] = dyy * hdx;
-    material<R>(P, c.lam, c.mu, H, N);
+    stress_n<R>(P, c, dxx, dxy, dyx, dyy, false, false, N);
 #pragma unroll
     for (int m = 0; m < 4; ++m) sn[F::n(m, i, j)] = N[m];
   };
@@ -1665,7 +1712,7 @@ __global__ void __launch_bounds__(M::NT) step_march_kernel(const Params P, const
     march_issue<M>(dsm, &bar[j % D], tm_g, tm_u, x0, y + 3, RB, gbase, y + 2, RB, ubase);
   };
 
-  const R kap = k.kap, hdx = k.hdx, scl = k.scl, lam = k.lam, mu = k.mu, sbx = k.sbx, sby = k.sby;
+  const R kap = k.kap, hdx = k.hdxs, scl = k.scl, sbx = k.sbxs, sby = k.sbys;
   const CollideK<R> &K = k.K;
   const size_t plane = (size_t)P.ny * P.pitch;
   gs *__restrict__ go = (gs *)S.g_out;
@@ -1692,14 +1739,10 @@ __global__ void __launch_bounds__(M::NT) step_march_kernel(const Params P, const
   auto phase_n2 = [&](int r0, int nrow) {
     for (int e = threadIdx.x; e < nrow * W1; e += NT) {
       const int row = r0 + e / W1, rx = e % W1, cx = rx + 1;
-      R dxx, dxy, dyx, dyy, H[4], Nn[4];
+      R dxx, dxy, dyx, dyy, Nn[4];
       udiff(U(row, cx + 1), U(row, cx - 1), dxx, dxy);
       udiff(U(row + 1, cx), U(row - 1, cx), dyx, dyy);
-      H[0] = dxx * hdx;
-      H[1] = dyx * hdx;
-      H[2] = dxy * hdx;
-      H[3] = dyy * hdx;
-      material<R>(P, lam, mu, H, Nn);
+      stress_n<R>(P, k, dxx, dxy, dyx, dyy, false, false, Nn);
 #pragma unroll
       for (int m = 0; m < 4; ++m) N(m, row, rx) = Nn[m];
     }
@@ -1924,7 +1967,8 @@ __global__ void __launch_bounds__(C::NT) init_kernel(const Params P, const Coef<
       const R eAe = R(ex(q) * ex(q)) * Axx + R(2 * ex(q) * ey(q)) * Axy + R(ey(q) * ey(q)) * Ayy;
       f[q] = wq<R>(q) * (rq + R(ex(q)) * jx + R(ey(q)) * jy + R(1.5) * eAe - R(0.5) * (Axx + Ayy)) * scl;
     }
-    collide<R>(f, Sx, Sy, c.K);
+    const R src = sizeof(R) == 8 ? c.K.s9 : R(1);
+    collide<R>(f, Sx * src, Sy * src, c.K);
     const size_t idx = (size_t)y * P.pitch + x;
     for (int q = 0; q < 9; ++q) gstore(g, q * plane + idx, f[q], scl);
     u[idx] = sm.u[ly + 2][lx + 2];

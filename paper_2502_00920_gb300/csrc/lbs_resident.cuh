@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(C::NT) resident_kernel(const Params P, const C
   const int x0 = (int)(blockIdx.x % ntx) * C::TX, y0 = (int)(blockIdx.x / ntx) * C::TY;
   const int plane = P.ny * P.pitch;
   const bool walls = !(P.per_x && P.per_y);
-  const R scl = c.scl, kap = c.kap, idx_ = c.idx, sbx = c.sbx, sby = c.sby, ics2 = c.ics2, cj = c.cj;
+  const R scl = c.scl, kap = c.kap, sbx = c.sbxs, sby = c.sbys, ics2 = c.ics2, cj = c.cj;
 
   // phase 1: this thread's node of R2
   const int e = threadIdx.x;
@@ -175,17 +175,14 @@ __global__ void __launch_bounds__(C::NT) resident_kernel(const Params P, const C
   const int r1x = e % C::R1W, r1y = e / C::R1W;
   int ux1 = 0, ux0 = 0, uy1 = 0, uy0 = 0, gx1 = x0 - 1 + r1x, gy1 = y0 - 1 + r1y;
   bool in1 = e < C::R1W * C::R1H && locate(P, gx1, gy1), keep1 = false;
-  R sx1 = 0, sy1 = 0;
+  bool onex1 = false, oney1 = false;
   if (in1) {
     int xa, xb, ya, yb;
-    bool onex, oney;
-    fd_taps<true>(P, r1x + 1, r1y + 1, gx1, gy1, xa, xb, ya, yb, onex, oney);
+    fd_taps<true>(P, r1x + 1, r1y + 1, gx1, gy1, xa, xb, ya, yb, onex1, oney1);
     ux1 = (r1y + 1) * C::R2W + xa;
     ux0 = (r1y + 1) * C::R2W + xb;
     uy1 = ya * C::R2W + r1x + 1;
     uy0 = yb * C::R2W + r1x + 1;
-    sx1 = onex ? idx_ : R(0.5) * idx_;
-    sy1 = oney ? idx_ : R(0.5) * idx_;
     keep1 = r1_own_node<C>(P, x0, y0, r1x, r1y) && (on_wall(P, gx1, gy1) || (LIN && P.extrap));
   }
   // phase 3: the own node's taps of N
@@ -199,8 +196,8 @@ __global__ void __launch_bounds__(C::NT) resident_kernel(const Params P, const C
     nx0 = (ry - 1) * C::R1W + xb;
     ny1 = ya * C::R1W + rx - 1;
     ny0 = yb * C::R1W + rx - 1;
-    sx2 = onex ? idx_ : R(0.5) * idx_;
-    sy2 = oney ? idx_ : R(0.5) * idx_;
+    sx2 = onex ? c.idxs : c.hdxs;
+    sy2 = oney ? c.idxs : c.hdxs;
   }
 
   R g0[9];
@@ -274,14 +271,10 @@ __global__ void __launch_bounds__(C::NT) resident_kernel(const Params P, const C
     }
     __syncthreads();
     if (in1) {
-      R H[4], N[4], dxx, dxy, dyx, dyy;
+      R N[4], dxx, dxy, dyx, dyy;
       udiff(su[ux1], su[ux0], dxx, dxy);
       udiff(su[uy1], su[uy0], dyx, dyy);
-      H[0] = dxx * sx1;
-      H[1] = dyx * sy1;
-      H[2] = dxy * sx1;
-      H[3] = dyy * sy1;
-      material<R>(P, c.lam, c.mu, H, N);
+      stress_n<R>(P, c, dxx, dxy, dyx, dyy, onex1, oney1, N);
 #pragma unroll
       for (int m = 0; m < 4; ++m) sn[m][e] = N[m];
       if (keep1) {
