@@ -224,8 +224,10 @@ def time_precision(L, I, torch, precision, n, steps, warmup, stream, v0dev, uref
     u = torch.empty((n, n, 2), dtype=torch.float64, device=v0dev.device)
     sim.fields_device(u, None, None)
     sim.sync()
-    sim.close()
     bpn = BYTES_PER_NODE[precision]
+    if L.tile_variant_name(precision, sim.variant) in ("step_fused2_tma_kernel", "step_column_kernel"):
+        bpn = bpn / 2  # two iterations per pass over the state (periodic lattice)
+    sim.close()
     out = {"mlups": n * n / (ms * 1e-3) / 1e6, "ms_per_step": ms, "gbs": bpn * n * n / (ms * 1e-3) / 1e9,
            "bytes_per_node": bpn, "iterations": warmup + steps}
     if uref is not None:
@@ -461,14 +463,13 @@ def main():
     # average duration in the timed region (events on the launching stream)
     peak, peak_kind = peaks()
     bpn = BYTES_PER_NODE[args.precision]
-    if L.tile_variant_name(args.precision, variant) == "step_fused2_tma_kernel":
+    if L.tile_variant_name(args.precision, variant) in ("step_fused2_tma_kernel", "step_column_kernel"):
         bpn = bpn / 2  # two iterations per pass over the state (periodic lattice)
     achieved = bpn * cells / (ms / K * 1e-3) / 1e9
     traffic = profile_traffic(args.precision, n)
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": traffic,
-                "kernel": f"{L.tile_variant_name(args.precision, variant)} + step_edge_kernel (one iteration, "
-                          f"tile variant {variant})",
+                "kernel": f"{L.tile_variant_name(args.precision, variant)} (tile variant {variant})",
                 "bytes_per_node": bpn, "peak_source": f"{peak_kind} hbm_gbs"}
     clocks = clk.summary()
     sim.close()

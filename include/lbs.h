@@ -245,7 +245,7 @@ int lbs_set_monitor_interval(lbs_handle *h, int64_t m);
 int lbs_set_graph_chunk(lbs_handle *h, int32_t k);
 
 /* Kernel tile variant (an index from lbs_tile_variants).  Each precision has a
- * default (the fastest on a large lattice); lbs_autotune picks per lattice. */
+ * default by the lattice's size and edges; lbs_autotune picks per lattice. */
 int lbs_set_variant(lbs_handle *h, int32_t variant);
 
 /* ---- checkpoint / resume (no counterpart in the paper) ------------------
@@ -320,9 +320,10 @@ int lbs_tile_variants(int32_t precision, int32_t *count, int32_t *tx, int32_t *t
 int lbs_tile_variant_kind(int32_t precision, int32_t variant);
 
 /* Name of the kernel that updates a variant's interior tiles (a static
- * string: "step_interior_kernel", "step_tma_kernel", "step_tma2_kernel" or
- * "step_march_kernel"; frame tiles always go to "step_edge_kernel"), or NULL
- * for an unknown precision or variant. */
+ * string: "step_interior_kernel", "step_tma_kernel", "step_tma2_kernel",
+ * "step_march_kernel", "step_fused2_tma_kernel" or "step_column_kernel"; frame
+ * tiles go to "step_edge_kernel"; the last two advance a periodic lattice by
+ * two iterations per launch), or NULL for an unknown precision or variant. */
 const char *lbs_tile_variant_name(int32_t precision, int32_t variant);
 
 /* ---- autotuner ---------------------------------------------------------- */

@@ -3,6 +3,7 @@
 
 #include "lbs_device.cuh"
 #include "lbs_batch.cuh"
+#include "lbs_column.cuh"
 #include "lbs_resident.cuh"
 
 namespace lbs {
@@ -17,8 +18,16 @@ using V4 = Cfg<P, 32, 16, 8>;
 using M6 = MarchCfg<V4, 8, 128, 2>;
 // 0-3: V0-V3 tiles read from global memory; 4: V4 tiles staged by TMA;
 // 5: V4 tiles, persistent blocks with a two-stage TMA ring; 6: row-marching
-// strips over the V4 tile columns; 7: V3 tiles staged by TMA
-constexpr int kVariants = 8;
+// strips over the V4 tile columns; 7: V3 tiles staged by TMA; 8: warp columns
+// (two iterations per launch on periodic lattices of even width, else one, with
+// V0 frame tiles)
+constexpr int kVariants = 9;
+// lattices from this many nodes on take variant 8 (us per iteration, variant 7
+// / 8; periodic, two iterations per launch: 1024^2 22.4 / 32.5, 1536^2 56.0 /
+// 48.5, 6000 x 400 55.9 / 50.2, 4096^2 236 / 210, 16384^2 3381 / 3001; walled:
+// 1021 x 509 18.9 / 33.2, 1500 x 1000 39.1 / 39.7, 400 x 5000 62.7 / 57.6, 2048^2
+// 83.3 / 72.7, 3000 x 1501 85.5 / 74.7, 4096^2 246 / 241, 6000 x 5000 419 / 417)
+constexpr int64_t kColumnNodes = 1 << 21;
 
 TileShape shape(int v) {
   switch (v) {
@@ -29,6 +38,7 @@ TileShape shape(int v) {
     case 4:
     case 5:
     case 6: return {V4::TX, V4::TY};
+    case 8: return {64, 64};
     default: return {V0::TX, V0::TY};
   }
 }
@@ -39,6 +49,7 @@ const char *name(int v) {
     case 5: return "step_tma2_kernel";
     case 6: return "step_march_kernel";
     case 7: return "step_tma_kernel";
+    case 8: return "step_column_kernel";
     default: return "step_interior_kernel";
   }
 }
@@ -52,6 +63,7 @@ cudaError_t step(const Params &p, const StepPtrs &s, int v, cudaStream_t st) {
     case 5: return launch_step_tma2<V4>(p, s, st);
     case 6: return launch_step_march<V4, M6>(p, s, st);
     case 7: return launch_step_tma<V3>(p, s, st);
+    case 8: return column_wraps(p) ? launch_column_periodic<P, 2>(p, s, st) : launch_step_column<V0>(p, s, st);
     default: return launch_step<V0>(p, s, st);
   }
 }
@@ -65,11 +77,19 @@ int kernels_per_step(const Params &p, int v) {
     case 4:
     case 5:
     case 6: return step_kernel_count<V4>(p);
+    case 8: return column_wraps(p) ? 1 : step_kernel_count<V0>(p);
     default: return step_kernel_count<V0>(p);
   }
 }
 
-int iterations_per_call(const Params &, int) { return 1; }
+int iterations_per_call(const Params &p, int v) { return v == 8 && column_wraps(p) ? 2 : 1; }
+
+cudaError_t step1(const Params &p, const StepPtrs &s, int, cudaStream_t st) {
+  return launch_column_periodic<P, 1>(p, s, st);
+}
+int kernels_per_step1(const Params &, int) { return 1; }
+
+int default_variant(const Params &p) { return (int64_t)p.nx * p.ny >= kColumnNodes ? 8 : 7; }
 
 bool tma_maps(const Params &p, int v, const void *g, const void *u, void *og, void *ou) {
   if (v == 6) return make_march_maps<V4, M6>(p, g, u, og, ou);
@@ -111,14 +131,14 @@ cudaError_t batch_step(int b, BatchLattice *lats, int nlats, const BatchTile *in
 
 const Launchers kL = {kVariants,
                       (1 << 4) | (1 << 5) | (1 << 6) | (1 << 7),
-                      7,  // default: the fastest on the 16384^2 roofline lattice
+                      default_variant,
                       shape,
                       name,
                       step,
                       kernels_per_step,
                       iterations_per_call,
-                      launch_step<V0>,
-                      step_kernel_count<V0>,
+                      step1,
+                      kernels_per_step1,
                       coef,
                       resident_applies,
                       resident,

@@ -3,6 +3,7 @@
 
 #include "lbs_device.cuh"
 #include "lbs_batch.cuh"
+#include "lbs_column.cuh"
 #include "lbs_resident.cuh"
 
 namespace lbs {
@@ -21,8 +22,15 @@ using V9 = Cfg<P, 32, 16, 16>;  // one node per thread, 512 threads
 // 5: V4 tiles, persistent blocks with a two-stage TMA ring; 6: row-marching
 // strips over the V4 tile columns; 7: V3 tiles staged by TMA; 8: V8 tiles
 // (four nodes per thread) read from global memory; 9: two fused iterations per
-// launch on V9 tiles (periodic lattices; one V0 iteration per call otherwise).
-constexpr int kVariants = 10;
+// launch on V9 tiles (periodic lattices; one V0 iteration per call otherwise);
+// 10: two iterations per launch in warp columns (periodic lattices of even
+// width; variant 4 otherwise).
+constexpr int kVariants = 11;
+// periodic lattices from this many nodes on take variant 10: below, too few
+// strips march to fill the GPU (us per iteration, variant 4 / 10: 512^2 12.9 /
+// 23.1, 1024^2 26.4 / 31.2, 1024 x 2048 45.3 / 44.0, 1536^2 48.9 / 48.4, 2048^2
+// 77.2 / 72.5, 400 x 6000 57.5 / 47.5, 4096^2 275 / 233, 16384^2 4204 / 3269)
+constexpr int64_t kColumnNodes = 1 << 21;
 
 TileShape shape(int v) {
   switch (v) {
@@ -35,6 +43,7 @@ TileShape shape(int v) {
     case 6: return {V4::TX, V4::TY};
     case 8: return {V8::TX, V8::TY};
     case 9: return {V9::TX, V9::TY};
+    case 10: return {64, 64};
     default: return {V0::TX, V0::TY};
   }
 }
@@ -46,8 +55,14 @@ const char *name(int v) {
     case 6: return "step_march_kernel";
     case 7: return "step_tma_kernel";
     case 9: return "step_fused2_tma_kernel";
+    case 10: return "step_column_kernel";
     default: return "step_interior_kernel";
   }
+}
+
+// one iteration on V4 tiles (variant 10 outside its lattices)
+cudaError_t step_single(const Params &p, const StepPtrs &s, cudaStream_t st) {
+  return s.tm_g ? launch_step_tma<V4>(p, s, st) : launch_step<V0>(p, s, st);
 }
 
 cudaError_t step(const Params &p, const StepPtrs &s, int v, cudaStream_t st) {
@@ -61,6 +76,7 @@ cudaError_t step(const Params &p, const StepPtrs &s, int v, cudaStream_t st) {
     case 7: return launch_step_tma<V3>(p, s, st);
     case 8: return launch_step<V8>(p, s, st);
     case 9: return fused2_applies(p) ? launch_step_fused2<V9>(p, s, st) : launch_step<V0>(p, s, st);
+    case 10: return column_wraps(p) ? launch_column_periodic<P, 2>(p, s, st) : step_single(p, s, st);
     default: return launch_step<V0>(p, s, st);
   }
 }
@@ -75,6 +91,7 @@ int kernels_per_step(const Params &p, int v) {
     case 5:
     case 6: return step_kernel_count<V4>(p);
     case 8: return step_kernel_count<V8>(p);
+    case 10: return column_wraps(p) ? 1 : step_kernel_count<V4>(p);
     case 9: {
       if (!fused2_applies(p)) return step_kernel_count<V0>(p);
       const int ntx = (p.nx + V9::TX - 1) / V9::TX, nty = (p.ny + V9::TY - 1) / V9::TY;
@@ -87,13 +104,24 @@ int kernels_per_step(const Params &p, int v) {
   }
 }
 
-int iterations_per_call(const Params &p, int v) { return v == 9 && fused2_applies(p) ? 2 : 1; }
+int iterations_per_call(const Params &p, int v) {
+  return (v == 9 && fused2_applies(p)) || (v == 10 && column_wraps(p)) ? 2 : 1;
+}
+
+cudaError_t step1(const Params &p, const StepPtrs &s, int v, cudaStream_t st) {
+  return v == 10 ? step_single(p, s, st) : launch_step<V0>(p, s, st);
+}
+int kernels_per_step1(const Params &p, int v) { return v == 10 ? step_kernel_count<V4>(p) : step_kernel_count<V0>(p); }
+
+int default_variant(const Params &p) {
+  return column_wraps(p) && (int64_t)p.nx * p.ny >= kColumnNodes ? 10 : 4;
+}
 
 bool tma_maps(const Params &p, int v, const void *g, const void *u, void *og, void *ou) {
   if (v == 9) return make_fused2_maps<V9>(p, g, u, og, ou);
   if (v == 6) return make_march_maps<V4, M6>(p, g, u, og, ou);
   if (v == 7) return make_tma_maps<V3>(p, g, u, og, ou);
-  if (v != 4 && v != 5) return false;
+  if (v != 4 && v != 5 && v != 10) return false;
   return make_tma_maps<V4>(p, g, u, og, ou);
 }
 
@@ -134,14 +162,14 @@ cudaError_t batch_step(int b, BatchLattice *lats, int nlats, const BatchTile *in
 
 const Launchers kL = {kVariants,
                       (1 << 4) | (1 << 5) | (1 << 6) | (1 << 7) | (1 << 9),
-                      4,  // default: the fastest on the 16384^2 roofline lattice
+                      default_variant,
                       shape,
                       name,
                       step,
                       kernels_per_step,
                       iterations_per_call,
-                      launch_step<V0>,
-                      step_kernel_count<V0>,
+                      step1,
+                      kernels_per_step1,
                       coef,
                       resident_applies,
                       resident,

@@ -54,6 +54,11 @@ int kernels_per_step(const Params &p, int v) {
 }
 
 int iterations_per_call(const Params &, int) { return 1; }
+cudaError_t step1(const Params &p, const StepPtrs &s, int v, cudaStream_t st) { return step(p, s, v, st); }
+int kernels_per_step1(const Params &p, int v) { return kernels_per_step(p, v); }
+
+// the fastest on the 4096^2 and 16384^2 periodic lattices
+int default_variant(const Params &) { return 3; }
 
 bool tma_maps(const Params &p, int v, const void *g, const void *u, void *og, void *ou) {
   if (v != 4) return false;
@@ -97,14 +102,14 @@ cudaError_t batch_step(int b, BatchLattice *lats, int nlats, const BatchTile *in
 
 const Launchers kL = {kVariants,
                       1 << 4,
-                      3,  // default: the fastest on the 16384^2 roofline lattice
+                      default_variant,
                       shape,
                       name,
                       step,
                       kernels_per_step,
                       iterations_per_call,
-                      launch_step<V0>,
-                      step_kernel_count<V0>,
+                      step1,
+                      kernels_per_step1,
                       coef,
                       resident_applies,
                       resident,

@@ -504,7 +504,7 @@ int lbs_create(const lbs_lattice *lat, const lbs_material *mat, const lbs_bcs *b
   h->zero_dev = h->kdev + 1;
   h->errdev = (int *)(h->kdev + 2);
   h->bytes = 2 * (s.g + s.u + s.b) + s.mon;
-  rc = select_variant(h, h->L->default_variant);
+  rc = select_variant(h, h->L->default_variant(h->P));
   // mon_out[7] holds the resident launches' barrier counters
   if (!rc && (cudaMemsetAsync(h->zero_dev, 0, 2 * sizeof(int64_t), h->stream) != cudaSuccess ||
               cudaMemsetAsync(h->mon_out + 7, 0, sizeof(double), h->stream) != cudaSuccess))
@@ -644,18 +644,20 @@ int lbs_step(lbs_handle *h, int64_t n) {
       n -= h->graph_chunk;
     } else {
       const int its = h->L->iterations_per_call(h->P, h->variant);
-      if (its > 1 && n >= its) {
+      // (a call of two does not step over an iteration at which a monitor is due)
+      const bool two = its > 1 && n >= its && !(h->mon_interval > 0 && h->k + 1 >= h->next_mon);
+      if (two) {
         LBS_CK(h->L->step(h->P, ptrs(h, h->parity, h->zero_dev, h->k), h->variant, h->stream));
         h->launches += h->L->kernels_per_step(h->P, h->variant);
       } else if (its > 1) {
-        // the last iteration of an odd count under a fused variant
-        LBS_CK(h->L->step1(h->P, ptrs(h, h->parity, h->zero_dev, h->k), h->stream));
-        h->launches += h->L->kernels_per_step1(h->P);
+        // a single iteration under a variant of two per call
+        LBS_CK(h->L->step1(h->P, ptrs(h, h->parity, h->zero_dev, h->k), h->variant, h->stream));
+        h->launches += h->L->kernels_per_step1(h->P, h->variant);
       } else {
         LBS_CK(h->L->step(h->P, ptrs(h, h->parity, h->zero_dev, h->k), h->variant, h->stream));
         h->launches += h->L->kernels_per_step(h->P, h->variant);
       }
-      const int done = (its > 1 && n >= its) ? its : 1;
+      const int done = two ? its : 1;
       h->parity ^= 1;
       h->k += done;
       n -= done;

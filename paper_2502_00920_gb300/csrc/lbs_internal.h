@@ -106,7 +106,7 @@ struct BatchTile {
 struct Launchers {
   int nvariants;
   int tma_mask;   // bit v set: variant v stages its interior tiles by TMA
-  int default_variant;
+  int (*default_variant)(const Params &p);  // the variant a new handle starts with
   TileShape (*shape)(int variant);
   const char *(*name)(int variant);  // the interior kernel of a variant, e.g. "step_tma_kernel"
   // one call of a variant: iterations_per_call iterations (2 for the fused
@@ -115,10 +115,10 @@ struct Launchers {
   cudaError_t (*step)(const Params &p, const StepPtrs &s, int variant, cudaStream_t st);
   int (*kernels_per_step)(const Params &p, int variant);
   int (*iterations_per_call)(const Params &p, int variant);
-  // exactly one iteration whatever the variant (global-memory tiles; the
-  // last iteration of an odd count under a fused variant); one or two kernels
-  cudaError_t (*step1)(const Params &p, const StepPtrs &s, cudaStream_t st);
-  int (*kernels_per_step1)(const Params &p);
+  // exactly one iteration under a variant of two per call (the last of an odd
+  // count); one or two kernels
+  cudaError_t (*step1)(const Params &p, const StepPtrs &s, int variant, cudaStream_t st);
+  int (*kernels_per_step1)(const Params &p, int variant);
   // the scheme's coefficients in the precision's compute type (Coef<real>) for
   // a batch's table (out: 32 doubles of room)
   void (*coef)(const Params &p, void *out);
