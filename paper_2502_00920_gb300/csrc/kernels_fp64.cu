@@ -110,6 +110,8 @@ const Launchers kL = {kVariants,
                       iterations_per_call,
                       step1,
                       kernels_per_step1,
+                      launch_edge_table<P::real>,
+                      launch_batch_edges<P::real>,
                       coef,
                       resident_applies,
                       resident,

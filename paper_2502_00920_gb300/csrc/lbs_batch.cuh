@@ -59,7 +59,7 @@ __device__ __forceinline__ void batch_walk(const BatchLattice *lats, const Batch
         sS.tm_g = sS.tm_u = nullptr;
         sS.err = err;
         sS.fork = nullptr;
-        sS.sev = L.sev ? L.sev + (size_t)it * 8 : nullptr;
+        sS.sev = L.sev ? (const char *)L.sev + (size_t)it * kEdgeStride : nullptr;
       }
     }
     __syncthreads();
@@ -89,6 +89,23 @@ template <class C>
 __global__ void __launch_bounds__(C::NT, 3) batch_frame3_kernel(const BatchLattice *lats, const BatchTile *tiles,
                                                                 int ntiles, int it, int *err) {
   batch_walk<C, true, false, false>(lats, tiles, ntiles, it, err);
+}
+
+// the edge tables of every lattice for the n iterations of the chunk, with the
+// frame tiles' own function: one thread per lattice, iteration and entry
+template <class R>
+__global__ void __launch_bounds__(128) batch_edges_kernel(BatchLattice *lats, int nlats, int n) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int per = n * kEdgeEntries;
+  if (i >= (int64_t)nlats * per) return;
+  const BatchLattice &L = lats[i / per];
+  if (L.sev) edge_table_entry<R>(L.P, L.k, L.sev, (int)(i % per));
+}
+template <class R>
+cudaError_t launch_batch_edges(BatchLattice *lats, int nlats, int n, cudaStream_t st) {
+  const int64_t m = (int64_t)nlats * n * kEdgeEntries;
+  if (m > 0) batch_edges_kernel<R><<<(unsigned)((m + 127) / 128), 128, 0, st>>>(lats, nlats, n);
+  return cudaGetLastError();
 }
 
 // resident blocks of a batch kernel on this device

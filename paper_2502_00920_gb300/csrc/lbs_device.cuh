@@ -284,6 +284,65 @@ __device__ inline void edge_value(const Params &P, int e, int64_t k, double out[
   out[1] = P.eamp[e][1] * f;
 }
 
+template <bool B, class X, class Y>
+struct Pick {
+  using type = X;
+};
+template <class X, class Y>
+struct Pick<false, X, Y> {
+  using type = Y;
+};
+
+// The prescribed values of one iteration as the wall rules read them: of the
+// four edges, then of the corners left-bottom, right-bottom, left-top,
+// right-top the mean of their two walls' values (Dirichlet on both).  In the
+// compute type, or in double for the two-point extrapolation (which takes the
+// mean itself).
+template <class R, bool LIN>
+using EdgeType = typename Pick<LIN, double, R>::type;
+constexpr int kEdgeEntries = 8;
+__device__ __forceinline__ int edge_corner(int xw, int yw) { return 4 + (xw == kRight ? 1 : 0) + (yw == kTop ? 2 : 0); }
+
+template <class T>
+__device__ inline void edge_entry(const Params &P, int i, int64_t k, T out[2]) {
+  double a[2], b[2];
+  if (i < 4) {
+    edge_value(P, i, k, a);
+  } else {
+    const int ex = kLeft + (i & 1), ey = kBottom + ((i >> 1) & 1);
+    if (P.etype[ex] != LBS_DIRICHLET || P.etype[ey] != LBS_DIRICHLET) return;
+    edge_value(P, ex, k, a);
+    edge_value(P, ey, k, b);
+    a[0] = 0.5 * (a[0] + b[0]);
+    a[1] = 0.5 * (a[1] + b[1]);
+  }
+  out[0] = (T)a[0];
+  out[1] = (T)a[1];
+}
+
+// a lattice's table of n iterations from k (one iteration every kEdgeStride bytes)
+template <class R>
+__device__ inline void edge_table_entry(const Params &P, int64_t k, void *sev, int i) {
+  char *row = (char *)sev + (size_t)(i / kEdgeEntries) * kEdgeStride;
+  const int e = i % kEdgeEntries;
+  if (P.extrap) {
+    if (e < 4) edge_entry(P, e, k + i / kEdgeEntries, ((double(*)[2])row)[e]);
+  } else {
+    edge_entry(P, e, k + i / kEdgeEntries, ((R(*)[2])row)[e]);
+  }
+}
+template <class R>
+__global__ void __launch_bounds__(128) edge_table_kernel(const Params P, const int64_t *kptr, int64_t koff, int n,
+                                                         void *sev) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n * kEdgeEntries) edge_table_entry<R>(P, *kptr + koff, sev, i);
+}
+template <class R>
+cudaError_t launch_edge_table(const Params &P, const int64_t *kptr, int64_t koff, int n, void *sev, cudaStream_t st) {
+  edge_table_kernel<R><<<(n * kEdgeEntries + 127) / 128, 128, 0, st>>>(P, kptr, koff, n, sev);
+  return cudaGetLastError();
+}
+
 // ------------------------------------------------------------------ boundary rules
 // Pull-form boundary rules at a wall node (x, y): for every direction q whose
 // source x - c_q dt lies outside the lattice (bit q of `mask`), the outgoing
@@ -322,7 +381,7 @@ __device__ __forceinline__ void wall_n(const Params &P, const R *bnd, int xw, in
   }
 }
 
-template <class R, class G, bool LIN, bool COH>
+template <class R, class G, bool COH>
 __device__ void wall_rules(const Params &P, const R *bnd, const G *g, const double (*sev)[2], int x, int y, int xw,
                            int yw, const R wn[4], const R g0[9], unsigned mask, R f[9], R ics2, R cj) {
   const bool xn = xw >= 0 && P.etype[xw] == LBS_NEUMANN;
@@ -357,7 +416,7 @@ __device__ void wall_rules(const Params &P, const R *bnd, const G *g, const doub
   // for the x wall (dX, nX) and the y wall (dY, nY) the node sits on (a
   // lattice without the setting has no second side-array layer to read).
   R dX[4] = {0, 0, 0, 0}, dY[4] = {0, 0, 0, 0}, nX[4] = {0, 0, 0, 0}, nY[4] = {0, 0, 0, 0};
-  if (LIN && P.extrap) {
+  if (P.extrap) {
     const size_t plane = (size_t)P.ny * P.pitch;
     const R own[4] = {r, Axx_o, Axy_o, Ayy_o};
 #pragma unroll
@@ -418,16 +477,8 @@ __device__ void wall_rules(const Params &P, const R *bnd, const G *g, const doub
         js[1] = sev[dxw ? xw : yw][1];
       }
       f[q] = g0[qb] + R(2) * wq<R>(q) * cj * (R(ex(q)) * (R)js[0] + R(ey(q)) * (R)js[1]);
-    } else if constexpr (!LIN) {
-      // Pi* of the wall(s) this link crosses
-      const R Axx = ox ? Axx_x : Axx_o;
-      const R Ayy = oy ? Ayy_y : Ayy_o;
-      const R Axy = (ox && oy) ? R(0.5) * (axy_x + axy_y) : (ox ? axy_x : axy_y);
-      const R e2 = R(ex(q) * ex(q) + ey(q) * ey(q));
-      const R eAe = R(ex(q) * ex(q)) * Axx + R(2 * ex(q) * ey(q)) * Axy + R(ey(q) * ey(q)) * Ayy;
-      f[q] = -g0[qb] + wq<R>(q) * (R(4) * r - R(3) * r * e2 + R(3) * eAe - (Axx + Ayy));
     } else {
-      // the same with the values extrapolated across the crossed walls only
+      // values extrapolated across the crossed walls only
       const R ax = ox ? R(1) : R(0), ay = oy ? R(1) : R(0);
       auto e = [&](int m, const R *a, const R *b) { return ax * a[m] + ay * b[m]; };
       const R rw = r + e(0, dX, dY);
@@ -440,6 +491,52 @@ __device__ void wall_rules(const Params &P, const R *bnd, const G *g, const doub
       const R e2 = R(ex(q) * ex(q) + ey(q) * ey(q));
       const R eAe = R(ex(q) * ex(q)) * Axx + R(2 * ex(q) * ey(q)) * Axy + R(ey(q) * ey(q)) * Ayy;
       f[q] = -g0[qb] + wq<R>(q) * (R(4) * rw - R(3) * rw * e2 + R(3) * eAe - (Axx + Ayy));
+    }
+  }
+}
+
+// The same rules with every node's own values (no extrapolation), on the
+// directions' masks: Tx, Ty are the prescribed values of the node's x and y
+// wall in the compute type, js their mean (a diagonal link between two
+// Dirichlet walls), and the sums leave out the terms whose factor e_a e_b is
+// zero.  (The general form above converts the values from double per node and
+// multiplies by the zeros; in FP64 those products are pipe slots.)
+template <class R>
+__device__ __forceinline__ void wall_rules_own(const Params &P, int xw, int yw, const R (*sev)[2], R ics2, R cj,
+                                               const R wn[4], const R g0[9], R f[9]) {
+  const unsigned crossx = crosses_x(xw), crossy = crosses_y(yw), mask = crossx | crossy;
+  const bool dirx = xw >= 0 && P.etype[xw] == LBS_DIRICHLET, diry = yw >= 0 && P.etype[yw] == LBS_DIRICHLET;
+  const R *Tx = sev[xw < 0 ? 0 : xw], *Ty = sev[yw < 0 ? 0 : yw], *js = sev[edge_corner(xw, yw)];
+  const R sgx = (xw == kRight) ? R(1) : R(-1), sgy = (yw == kTop) ? R(1) : R(-1);
+  R r = 0, mxx = 0, mxy = 0, myy = 0;
+#pragma unroll
+  for (int q = 0; q < 9; ++q) {
+    r += g0[q];
+    if (ex(q) != 0) mxx += g0[q];
+    if (ex(q) * ey(q) != 0) mxy += R(ex(q) * ey(q)) * g0[q];
+    if (ey(q) != 0) myy += g0[q];
+  }
+  const R Axx_o = R(3) * mxx, Ayy_o = R(3) * myy;
+  const R Axx_x = (wn[0] - sgx * Tx[0]) * ics2, axy_x = (wn[1] - sgx * Tx[1]) * ics2;
+  const R Ayy_y = (wn[2] - sgy * Ty[1]) * ics2, axy_y = (wn[3] - sgy * Ty[0]) * ics2;
+#pragma unroll
+  for (int q = 1; q < 9; ++q) {
+    if (!(mask & (1u << q))) continue;
+    const bool ox = ex(q) != 0 && (crossx & (1u << q)), oy = ey(q) != 0 && (crossy & (1u << q));
+    const bool dxw = ox && dirx, dyw = oy && diry;
+    if (dxw || dyw) {
+      const R *j = dxw && dyw ? js : (dxw ? Tx : Ty);
+      f[q] = g0[opp(q)] + R(2) * wq<R>(q) * cj * (R(ex(q)) * j[0] + R(ey(q)) * j[1]);
+    } else {
+      const R Axx = ox ? Axx_x : Axx_o;
+      const R Ayy = oy ? Ayy_y : Ayy_o;
+      if (ex(q) * ey(q) == 0) {
+        f[q] = -g0[opp(q)] + wq<R>(q) * (R(4) * r - R(3) * r + R(3) * (ex(q) != 0 ? Axx : Ayy) - (Axx + Ayy));
+      } else {
+        const R Axy = (ox && oy) ? R(0.5) * (axy_x + axy_y) : (ox ? axy_x : axy_y);
+        const R eAe = Axx + R(2 * ex(q) * ey(q)) * Axy + Ayy;
+        f[q] = -g0[opp(q)] + wq<R>(q) * (R(4) * r - R(3) * r * R(2) + R(3) * eAe - (Axx + Ayy));
+      }
     }
   }
 }
@@ -647,8 +744,9 @@ struct TileCfg : TileGeom<TX_, TY_, NTY_> {
 // LIN: the two-point wall extrapolation (lattices with P.extrap set).
 template <class Pr, bool EDGE, bool LIN, bool COH = false>
 __device__ __forceinline__ void gather(const Params &P, const typename Pr::gs *g, const typename Pr::real *bnd,
-                                       const double (*sev)[2], int x, int y, const Coef<typename Pr::real> &k,
-                                       typename Pr::real f[9], typename Pr::real &gx, typename Pr::real &gy) {
+                                       const EdgeType<typename Pr::real, LIN> (*sev)[2], int x, int y,
+                                       const Coef<typename Pr::real> &k, typename Pr::real f[9],
+                                       typename Pr::real &gx, typename Pr::real &gy) {
   using R = typename Pr::real;
   const size_t plane = (size_t)P.ny * P.pitch;
   const size_t idx = (size_t)y * P.pitch + x;
@@ -663,56 +761,27 @@ __device__ __forceinline__ void gather(const Params &P, const typename Pr::gs *g
 #pragma unroll
     for (int q = 1; q < 9; ++q) g0[q] = gld<COH>(g, q * plane + idx, inv);
     g0[0] = 0;
-  } else if constexpr (sizeof(R) == 8 && !COH) {
-    // FP64: loads between the branches (the batched form below takes the
-    // frame kernel past 128 registers, halving its blocks per SM)
-    unsigned mask = 0;
-#pragma unroll
-    for (int q = 0; q < 9; ++q) {
-      g0[q] = gload(g, q * plane + idx, inv);
-      int sx, sy;
-      if (!stream_source(P, x, y, q, sx, sy)) {
-        mask |= 1u << q;
-        f[q] = 0;
-      } else {
-        f[q] = gload(g, q * plane + (size_t)sy * P.pitch + sx, inv);
-      }
-    }
-    if (mask) {
-      int xw, yw;
-      R wn[4];
-      walls_of(P, x, y, xw, yw);
-      wall_n<COH>(P, bnd, xw, yw, x, y, wn);
-      wall_rules<R, typename Pr::gs, LIN, COH>(P, bnd, g, sev, x, y, xw, yw, wn, g0, mask, f, k.ics2, k.cj);
-    }
   } else {
-    // source of each population first (the node itself where the source
-    // lies outside the lattice), then all eighteen loads without branches in
-    // between, so that they are in flight together
-    unsigned mask = 0;
-    size_t src[9];
-    int xw, yw;
-    R wn[4];
+    // all loads without branches in between, so that they are in flight
+    // together; what a wall supplies is overwritten by the rules
+    int xb, xf, yb, yf, xw, yw;
+    stream_sides(x, P.nx, P.per_x, xb, xf);
+    stream_sides(y, P.ny, P.per_y, yb, yf);
     walls_of(P, x, y, xw, yw);
-    if constexpr (COH) wall_n<COH>(P, bnd, xw, yw, x, y, wn);  // (in flight with the populations)
+    R wn[4];
+    wall_n<COH>(P, bnd, xw, yw, x, y, wn);
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
-      int sx, sy;
-      const bool in = stream_source(P, x, y, q, sx, sy);
-      if (!in) mask |= 1u << q;
-      src[q] = in ? (size_t)sy * P.pitch + sx : idx;
-    }
-#pragma unroll
-    for (int q = 0; q < 9; ++q) {
+      const int sx = ex(q) > 0 ? xb : (ex(q) < 0 ? xf : x), sy = ey(q) > 0 ? yb : (ey(q) < 0 ? yf : y);
       g0[q] = gld<COH>(g, q * plane + idx, inv);
-      f[q] = gld<COH>(g, q * plane + src[q], inv);
+      f[q] = gld<COH>(g, q * plane + (size_t)sy * P.pitch + sx, inv);
     }
-#pragma unroll
-    for (int q = 0; q < 9; ++q)
-      if (mask & (1u << q)) f[q] = 0;
-    if (mask) {
-      if constexpr (!COH) wall_n<COH>(P, bnd, xw, yw, x, y, wn);
-      wall_rules<R, typename Pr::gs, LIN, COH>(P, bnd, g, sev, x, y, xw, yw, wn, g0, mask, f, k.ics2, k.cj);
+    if (xw >= 0 || yw >= 0) {
+      if constexpr (LIN)
+        wall_rules<R, typename Pr::gs, COH>(P, bnd, g, sev, x, y, xw, yw, wn, g0, crosses_x(xw) | crosses_y(yw),
+                                                 f, k.ics2, k.cj);
+      else
+        wall_rules_own<R>(P, xw, yw, sev, k.ics2, k.cj, wn, g0, f);
     }
   }
   first_moment(g0, gx, gy);
@@ -827,17 +896,16 @@ __device__ __forceinline__ void step_tile(const Params &P, const Coef<typename C
   const us *__restrict__ u = (const us *)S.u_in;
   us *__restrict__ uo = (us *)S.u_out;
   const R *bnd = (const R *)S.b_in;
-  const int64_t k = EDGE ? (*S.kptr + S.koff) : 0;
-  // boundary values of the four edges at iteration k, evaluated once per
-  // tile (the wall rules of every wall node read them)
-  __shared__ double sev[4][2];
-  if (EDGE) {
-    if (S.sev) {
-      if (threadIdx.x < 8) sev[threadIdx.x >> 1][threadIdx.x & 1] = S.sev[threadIdx.x];
-    } else if (threadIdx.x < 4) {
-      edge_value(P, threadIdx.x, k, sev[threadIdx.x]);
-    }
+  const int64_t k = EDGE && !S.sev ? (*S.kptr + S.koff) : 0;
+  // the edges' prescribed values at this iteration: from the launch's table, or
+  // evaluated here once per tile
+  using T = EdgeType<R, LIN>;
+  __shared__ T sevs[EDGE ? kEdgeEntries : 1][2];
+  const T(*sev)[2] = (const T(*)[2])S.sev;
+  if (EDGE && !sev) {
+    if (threadIdx.x < (LIN ? 4 : kEdgeEntries)) edge_entry<T>(P, threadIdx.x, k, sevs[threadIdx.x]);
     __syncthreads();
+    sev = sevs;
   }
   const int tx = threadIdx.x % C::TX, ty = threadIdx.x / C::TX;
 

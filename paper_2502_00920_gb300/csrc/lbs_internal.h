@@ -58,9 +58,13 @@ struct StepPtrs {
   const void *tm_u;     //   u_in (TMA tile variants only)
   int *err;             // device flag set when a bounded wait gives up
   const StreamFork *fork;  // host: run the frame tiles beside the interior tiles (or null)
-  const double *sev;    // the four edges' prescribed values at this iteration ([4][2],
-                        //   device), or null: the frame tiles evaluate them
+  const void *sev;      // the edges' prescribed values at this iteration (a row of an
+                        //   edge table, device), or null: the frame tiles evaluate them
 };
+
+// Edge tables: one row of kEdgeStride bytes per iteration (edge_table_entry in
+// lbs_device.cuh); a handle keeps one of kEdgeBatch iterations.
+constexpr int kEdgeStride = 128, kEdgeBatch = 64;
 
 // Device pointers of one lattice for a resident launch: both buffers of each
 // state array, the barrier's two counters (zero between launches) and the
@@ -85,14 +89,13 @@ struct BatchLattice {
                  // chunk steps iteration k + it, buffers [(k + it) & 1]); advanced
                  // on the device once per chunk (launch_batch_advance)
   int64_t kend;  // the lattice stops here (its tiles return at once)
-  double *sev;   // the edges' prescribed values for the iterations of the chunk,
-                 // [it][4][2] (filled once per chunk, launch_batch_edges)
+  void *sev;     // edge table of the chunk's iterations (filled once per chunk,
+                 // Launchers::batch_edges)
 };
 
 // advance every lattice's chunk-start iteration by a chunk of n launches
 // (to its end at most); one launch
 cudaError_t launch_batch_advance(BatchLattice *lats, int nlats, int n, cudaStream_t st);
-cudaError_t launch_batch_edges(BatchLattice *lats, int nlats, int n, cudaStream_t st);
 
 // One tile of a batch: lattice index and tile coordinates (in tiles).
 struct BatchTile {
@@ -119,6 +122,10 @@ struct Launchers {
   // count); one or two kernels
   cudaError_t (*step1)(const Params &p, const StepPtrs &s, int variant, cudaStream_t st);
   int (*kernels_per_step1)(const Params &p, int variant);
+  // edge tables: n iterations from *kptr + koff of one lattice; the n
+  // iterations of a chunk of every lattice of a batch
+  cudaError_t (*edges)(const Params &p, const int64_t *kptr, int64_t koff, int n, void *sev, cudaStream_t st);
+  cudaError_t (*batch_edges)(BatchLattice *lats, int nlats, int n, cudaStream_t st);
   // the scheme's coefficients in the precision's compute type (Coef<real>) for
   // a batch's table (out: 32 doubles of room)
   void (*coef)(const Params &p, void *out);
@@ -204,6 +211,7 @@ struct lbs_handle {
   size_t bytes;
   int cfl_warn;
   int64_t launches;         // kernels launched for this handle
+  void *sev;                // edge table of kEdgeBatch iterations
   int *errdev;              // device flag: a bounded wait in a kernel gave up
   CUtensorMap tm_g[2];      // TMA descriptors of g[0], g[1] and u[0], u[1]
   CUtensorMap tm_u[2];      //   for the current variant (TMA variants only)

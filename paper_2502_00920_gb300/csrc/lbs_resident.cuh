@@ -46,56 +46,6 @@ __device__ __forceinline__ bool grid_barrier(unsigned *count, unsigned target, i
   return __syncthreads_and(ok) != 0;
 }
 
-// The own-value wall rules of wall_rules() for one node with what does not
-// change between iterations taken out: sev holds the edges' values in the
-// compute type, js the momentum of a diagonal link between two Dirichlet walls
-// (their mean), and the sums leave out the terms whose factor e_a e_b is zero.
-template <class R>
-__device__ __forceinline__ void wall_rules_own(unsigned mask, unsigned crossx, unsigned crossy, bool dirx, bool diry,
-                                               R sgx, R sgy, R ics2, R cj, const R wn[4], const R *Tx, const R *Ty,
-                                               const R *js, const R g0[9], R f[9]) {
-  R r = 0, mxx = 0, mxy = 0, myy = 0;
-#pragma unroll
-  for (int q = 0; q < 9; ++q) {
-    r += g0[q];
-    if (ex(q) != 0) mxx += g0[q];
-    if (ex(q) * ey(q) != 0) mxy += R(ex(q) * ey(q)) * g0[q];
-    if (ey(q) != 0) myy += g0[q];
-  }
-  const R Axx_o = R(3) * mxx, Ayy_o = R(3) * myy;
-  const R Axx_x = (wn[0] - sgx * Tx[0]) * ics2, axy_x = (wn[1] - sgx * Tx[1]) * ics2;
-  const R Ayy_y = (wn[2] - sgy * Ty[1]) * ics2, axy_y = (wn[3] - sgy * Ty[0]) * ics2;
-#pragma unroll
-  for (int q = 1; q < 9; ++q) {
-    if (!(mask & (1u << q))) continue;
-    const bool ox = ex(q) != 0 && (crossx & (1u << q)), oy = ey(q) != 0 && (crossy & (1u << q));
-    const bool dxw = ox && dirx, dyw = oy && diry;
-    if (dxw || dyw) {
-      const R *j = dxw && dyw ? js : (dxw ? Tx : Ty);
-      f[q] = g0[opp(q)] + R(2) * wq<R>(q) * cj * (R(ex(q)) * j[0] + R(ey(q)) * j[1]);
-    } else {
-      const R Axx = ox ? Axx_x : Axx_o;
-      const R Ayy = oy ? Ayy_y : Ayy_o;
-      if (ex(q) * ey(q) == 0) {
-        f[q] = -g0[opp(q)] + wq<R>(q) * (R(4) * r - R(3) * r + R(3) * (ex(q) != 0 ? Axx : Ayy) - (Axx + Ayy));
-      } else {
-        const R Axy = (ox && oy) ? R(0.5) * (axy_x + axy_y) : (ox ? axy_x : axy_y);
-        const R eAe = Axx + R(2 * ex(q) * ey(q)) * Axy + Ayy;
-        f[q] = -g0[opp(q)] + wq<R>(q) * (R(4) * r - R(3) * r * R(2) + R(3) * eAe - (Axx + Ayy));
-      }
-    }
-  }
-}
-
-template <bool B, class X, class Y>
-struct Pick {
-  using type = X;
-};
-template <class X, class Y>
-struct Pick<false, X, Y> {
-  using type = Y;
-};
-
 // iterations whose edge values are evaluated at once
 constexpr int kSevBatch = 32;
 
@@ -116,11 +66,10 @@ __global__ void __launch_bounds__(C::NT) resident_kernel(const Params P, const C
   using gs = typename C::gs;
   using us = typename C::us;
   using R = typename C::real;
-  using T = typename Pick<LIN, double, R>::type;  // edge values: the linear reading takes them in double
+  using T = EdgeType<R, LIN>;
   __shared__ us su[C::R2H * C::R2W];
   __shared__ R sn[4][C::R1H * C::R1W];
-  // per iteration: the four edges' values, then the four corners' means
-  __shared__ T sev[kSevBatch][8][2];
+  __shared__ T sev[kSevBatch][kEdgeEntries][2];
   int bad = 0;
   if (threadIdx.x == 0) bad = *(volatile int *)S.err;
   if (__syncthreads_or(bad)) return;
@@ -134,7 +83,6 @@ __global__ void __launch_bounds__(C::NT) resident_kernel(const Params P, const C
   const int e = threadIdx.x;
   int rx = 0, ry = 0, x = 0, y = 0, idx = 0, src[9], xw = -1, yw = -1;
   bool in = false, own = false;
-  unsigned mask = 0, crossx = 0, crossy = 0;
   us uu;
   if (e < C::OWN + C::NRING) {
     if (e < C::OWN) {
@@ -152,24 +100,17 @@ __global__ void __launch_bounds__(C::NT) resident_kernel(const Params P, const C
   if (in) {
     idx = y * P.pitch + x;
     walls_of(P, x, y, xw, yw);
+    int xb, xf, yb, yf;
+    stream_sides(x, P.nx, P.per_x, xb, xf);
+    stream_sides(y, P.ny, P.per_y, yb, yf);
 #pragma unroll
-    for (int q = 0; q < 9; ++q) {
-      int sx, sy;
-      bool ox, oy;
-      const bool inside = stream_source(P, x, y, q, sx, sy);
-      link_crosses(P, x, y, q, ox, oy);
-      if (!inside) mask |= 1u << q;
-      if (ox) crossx |= 1u << q;
-      if (oy) crossy |= 1u << q;
-      src[q] = q * plane + (inside ? sy * P.pitch + sx : idx);
-    }
+    for (int q = 0; q < 9; ++q)
+      src[q] = q * plane + (ey(q) > 0 ? yb : (ey(q) < 0 ? yf : y)) * P.pitch +
+               (ex(q) > 0 ? xb : (ex(q) < 0 ? xf : x));
     uu = ld_coh((const us *)S.u[parity] + idx);
   }
   const bool nx_ = xw >= 0 && P.etype[xw] == LBS_NEUMANN, ny_ = yw >= 0 && P.etype[yw] == LBS_NEUMANN;
   const int wx_at = nx_ ? (int)side_entry(P, 0, xw, y) : 0, wy_at = ny_ ? (int)side_entry(P, 0, yw, x) : 0;
-  const bool dirx = xw >= 0 && P.etype[xw] == LBS_DIRICHLET, diry = yw >= 0 && P.etype[yw] == LBS_DIRICHLET;
-  const R sgx = (xw == kRight) ? R(1) : R(-1), sgy = (yw == kTop) ? R(1) : R(-1);
-  const int corner = 4 + (xw == kRight ? 1 : 0) + (yw == kTop ? 2 : 0);
 
   // phase 2: this thread's node of R1 and its taps of u
   const int r1x = e % C::R1W, r1y = e / C::R1W;
@@ -221,46 +162,23 @@ __global__ void __launch_bounds__(C::NT) resident_kernel(const Params P, const C
 #pragma unroll
         for (int q = 0; q < 9; ++q) g0[q] = half_wide(ld_coh(g + (q * plane + idx)));
       }
-      if (mask) {
-#pragma unroll
-        for (int q = 0; q < 9; ++q)
-          if (mask & (1u << q)) f[q] = 0;
-      }
     }
     if (walls && it % kSevBatch == 0) {
       // (while the populations are in flight)
-      for (int j = threadIdx.x; j < kSevBatch * 4; j += C::NT) {
-        double v[2];
-        if (it + j / 4 < n) {
-          edge_value(P, j % 4, k0 + it + j / 4, v);
-          sev[j / 4][j % 4][0] = (T)v[0];
-          sev[j / 4][j % 4][1] = (T)v[1];
-        }
-      }
-      if constexpr (!LIN) {
-        for (int j = threadIdx.x; j < kSevBatch * 4; j += C::NT) {
-          double a[2], b[2];
-          if (it + j / 4 < n && P.etype[kLeft + j % 2] == LBS_DIRICHLET &&
-              P.etype[kBottom + j % 4 / 2] == LBS_DIRICHLET) {
-            edge_value(P, kLeft + j % 2, k0 + it + j / 4, a);
-            edge_value(P, kBottom + j % 4 / 2, k0 + it + j / 4, b);
-            sev[j / 4][4 + j % 4][0] = (T)(0.5 * (a[0] + b[0]));
-            sev[j / 4][4 + j % 4][1] = (T)(0.5 * (a[1] + b[1]));
-          }
-        }
-      }
+      constexpr int E = LIN ? 4 : kEdgeEntries;
+      for (int j = threadIdx.x; j < kSevBatch * E; j += C::NT)
+        if (it + j / E < n) edge_entry<T>(P, j % E, k0 + it + j / E, sev[j / E][j % E]);
       __syncthreads();
     }
     if (in) {
-      if (mask) {
-        const auto *ev = sev[it % kSevBatch];
+      if (xw >= 0 || yw >= 0) {
         if constexpr (LIN) {
           R wnl[4];
           wall_n<true>(P, bnd, xw, yw, x, y, wnl);
-          wall_rules<R, gs, true, true>(P, bnd, g, ev, x, y, xw, yw, wnl, g0, mask, f, ics2, cj);
+          wall_rules<R, gs, true>(P, bnd, g, sev[it % kSevBatch], x, y, xw, yw, wnl, g0, crosses_x(xw) | crosses_y(yw),
+                                  f, ics2, cj);
         } else {
-          wall_rules_own<R>(mask, crossx, crossy, dirx, diry, sgx, sgy, ics2, cj, wn, ev[xw < 0 ? 0 : xw],
-                            ev[yw < 0 ? 0 : yw], ev[corner], g0, f);
+          wall_rules_own<R>(P, xw, yw, sev[it % kSevBatch], ics2, cj, wn, g0, f);
         }
       }
       R gmx, gmy, fmx, fmy;

@@ -99,6 +99,20 @@ LBS_HD bool stream_source(const G &P, int x, int y, int q, int &sx, int &sy) {
   return in;
 }
 
+// The neighbour one step back and forward along an axis of n nodes: wrapped on
+// a periodic axis, the node itself beyond a wall (there the boundary rules
+// supply what would stream in).
+LBS_HD void stream_sides(int x, int n, int per, int &back, int &fwd) {
+  back = x > 0 ? x - 1 : (per ? n - 1 : x);
+  fwd = x < n - 1 ? x + 1 : (per ? 0 : x);
+}
+
+// The directions q whose streaming source lies beyond the x wall xw / the y
+// wall yw (-1: none) the node is on, as bit masks: as link_crosses, for all
+// q at once.
+LBS_HD unsigned crosses_x(int xw) { return xw == kLeft ? 0x122u : (xw == kRight ? 0x0c8u : 0u); }
+LBS_HD unsigned crosses_y(int yw) { return yw == kBottom ? 0x064u : (yw == kTop ? 0x190u : 0u); }
+
 // Whether the outgoing link opp(q) of node (x, y) crosses the x wall (ox) or
 // the y wall (oy): exactly the directions q whose source stream_source finds
 // beyond a wall.
