@@ -508,6 +508,41 @@ __device__ __forceinline__ void wall_rules_own(const Params &P, int xw, int yw, 
   const bool dirx = xw >= 0 && P.etype[xw] == LBS_DIRICHLET, diry = yw >= 0 && P.etype[yw] == LBS_DIRICHLET;
   const R *Tx = sev[xw < 0 ? 0 : xw], *Ty = sev[yw < 0 ? 0 : yw], *js = sev[edge_corner(xw, yw)];
   const R sgx = (xw == kRight) ? R(1) : R(-1), sgy = (yw == kTop) ? R(1) : R(-1);
+  if constexpr (sizeof(R) == 8) {
+    // FP64: the moments from pair sums, and the rule with its sums collected.
+    // With t = Axx + Ayy, an axis link along x sees r + 2 Axx - Ayy (along y
+    // r + 2 Ayy - Axx), a diagonal one 2 (t - r +- 3 Axy): about 30 pipe slots a
+    // wall node where the sums as written take 70 (a wall node's warp is the
+    // longest chain of a small lattice's iteration).
+    const R s57 = g0[5] + g0[7], s68 = g0[6] + g0[8], sd = s57 + s68;
+    const R s13 = g0[1] + g0[3], s24 = g0[2] + g0[4];
+    const R mxx = s13 + sd, myy = s24 + sd, r = g0[0] + (mxx + s24);
+    const R i2 = ics2;
+    const R Axx_x = fmr(wn[0], i2, -(sgx * (Tx[0] * i2))), axy_x = fmr(wn[1], i2, -(sgx * (Tx[1] * i2)));
+    const R Ayy_y = fmr(wn[2], i2, -(sgy * (Ty[1] * i2))), axy_y = fmr(wn[3], i2, -(sgy * (Ty[0] * i2)));
+#pragma unroll
+    for (int q = 1; q < 9; ++q) {
+      if (!(mask & (1u << q))) continue;
+      const bool ox = ex(q) != 0 && (crossx & (1u << q)), oy = ey(q) != 0 && (crossy & (1u << q));
+      const bool dxw = ox && dirx, dyw = oy && diry;
+      if (dxw || dyw) {
+        const R *j = dxw && dyw ? js : (dxw ? Tx : Ty);
+        const R ej = ex(q) * ey(q) == 0 ? (ex(q) != 0 ? R(ex(q)) * j[0] : R(ey(q)) * j[1])
+                                        : R(ex(q)) * j[0] + R(ey(q)) * j[1];
+        f[q] = fmr(R(2) * wq<R>(q) * cj, ej, g0[opp(q)]);
+      } else {
+        const R Axx = ox ? Axx_x : R(3) * mxx;
+        const R Ayy = oy ? Ayy_y : R(3) * myy;
+        if (ex(q) * ey(q) == 0) {
+          f[q] = fmr(wq<R>(q), ex(q) != 0 ? fmr(R(2), Axx, r - Ayy) : fmr(R(2), Ayy, r - Axx), -g0[opp(q)]);
+        } else {
+          const R Axy = (ox && oy) ? R(0.5) * (axy_x + axy_y) : (ox ? axy_x : axy_y);
+          f[q] = fmr(R(2) * wq<R>(q), fmr(R(3 * ex(q) * ey(q)), Axy, (Axx + Ayy) - r), -g0[opp(q)]);
+        }
+      }
+    }
+    return;
+  }
   R r = 0, mxx = 0, mxy = 0, myy = 0;
 #pragma unroll
   for (int q = 0; q < 9; ++q) {
