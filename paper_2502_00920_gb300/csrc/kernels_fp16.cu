@@ -28,6 +28,8 @@ constexpr int kVariants = 9;
 // 1021 x 509 18.9 / 33.2, 1500 x 1000 39.1 / 39.7, 400 x 5000 62.7 / 57.6, 2048^2
 // 83.3 / 72.7, 3000 x 1501 85.5 / 74.7, 4096^2 246 / 241, 6000 x 5000 419 / 417)
 constexpr int64_t kColumnNodes = 1 << 21;
+// lines of default_variant
+constexpr int64_t kSmallNodes = 400000, kWaveNodes = 800000;
 
 TileShape shape(int v) {
   switch (v) {
@@ -89,7 +91,19 @@ cudaError_t step1(const Params &p, const StepPtrs &s, int, cudaStream_t st) {
 }
 int kernels_per_step1(const Params &, int) { return 1; }
 
-int default_variant(const Params &p) { return (int64_t)p.nx * p.ny >= kColumnNodes ? 8 : 7; }
+// Below the columns, by size and edges; us per iteration, one lattice alone /
+// three side by side.  Small lattices pull from global memory (walled 300^2
+// variant 0 6.8 / 3.0, 7 11.6 / 3.6; 512^2 7.9 / 5.3, 15.4 / 5.4). Walled ones of
+// several waves take the smaller TMA tiles, which leave fewer nodes to the frame
+// tiles (4096 x 256 variant 4 22.1 / 18.6, 7 27.0 / 25.0; 1500 x 1300 38.3 / 32.5,
+// 47.3 / 36.3); the rest the larger (1021 x 509 variant 4 14.9 / 9.7, 7 16.4 / 9.5;
+// 1024^2 periodic 23.0 / 18.5, 21.6 / 17.8).
+int default_variant(const Params &p) {
+  const int64_t nodes = (int64_t)p.nx * p.ny;
+  if (nodes >= kColumnNodes) return 8;
+  if (nodes < kSmallNodes) return 0;
+  return nodes >= kWaveNodes && !(p.per_x && p.per_y) ? 4 : 7;
+}
 
 bool tma_maps(const Params &p, int v, const void *g, const void *u, void *og, void *ou) {
   if (v == 6) return make_march_maps<V4, M6>(p, g, u, og, ou);

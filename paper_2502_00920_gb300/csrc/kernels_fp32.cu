@@ -31,6 +31,8 @@ constexpr int kVariants = 11;
 // 23.1, 1024^2 26.4 / 31.2, 1024 x 2048 45.3 / 44.0, 1536^2 48.9 / 48.4, 2048^2
 // 77.2 / 72.5, 400 x 6000 57.5 / 47.5, 4096^2 275 / 233, 16384^2 4204 / 3269)
 constexpr int64_t kColumnNodes = 1 << 21;
+// lattices below this many nodes default to variant 0 (see default_variant)
+constexpr int64_t kSmallNodes = 400000;
 
 TileShape shape(int v) {
   switch (v) {
@@ -113,8 +115,14 @@ cudaError_t step1(const Params &p, const StepPtrs &s, int v, cudaStream_t st) {
 }
 int kernels_per_step1(const Params &p, int v) { return v == 10 ? step_kernel_count<V4>(p) : step_kernel_count<V0>(p); }
 
+// Small lattices (a wave of tiles or less: every launch is one tile's latency)
+// pull from global memory, where a tile starts without waiting for its boxes;
+// us per iteration, one lattice alone / three side by side, variant 0 against 4:
+// 300^2 walled 6.7 / 2.9 against 7.5 / 3.0, 512^2 7.7 / 5.7 against 13.2 / 5.6, 1021
+// x 509 13.2 / 12.7 against 15.5 / 11.5, 1024^2 26.5 / 25.0 against 26.5 / 20.7.
 int default_variant(const Params &p) {
-  return column_wraps(p) && (int64_t)p.nx * p.ny >= kColumnNodes ? 10 : 4;
+  const int64_t nodes = (int64_t)p.nx * p.ny;
+  return column_wraps(p) && nodes >= kColumnNodes ? 10 : (nodes < kSmallNodes ? 0 : 4);
 }
 
 bool tma_maps(const Params &p, int v, const void *g, const void *u, void *og, void *ou) {
