@@ -207,6 +207,28 @@ static Sizes sizes_of(const Params &p, const Launchers &L) {
   return s;
 }
 
+// Places of the buffers in one block: each starts on a 256-byte boundary.  (One
+// allocation and one release per handle: seven of each took most of the 0.4 ms
+// that creating and destroying a handle cost, which a server pays per request.)
+struct Layout {
+  size_t g[2], u[2], b[2], mon, total;
+};
+static Layout layout_of(const Sizes &s) {
+  Layout l;
+  size_t at = 0;
+  auto take = [&](size_t bytes) {
+    const size_t p = at;
+    at += (bytes + 255) / 256 * 256;
+    return p;
+  };
+  for (int i = 0; i < 2; ++i) l.g[i] = take(s.g);
+  for (int i = 0; i < 2; ++i) l.u[i] = take(s.u);
+  for (int i = 0; i < 2; ++i) l.b[i] = take(s.b);
+  l.mon = take(s.mon);
+  l.total = at;
+  return l;
+}
+
 // Device room for host transfers without allocating: the g and u buffers of
 // the parity the state is not in.  The next iteration overwrites them without
 // reading them, so set_initial stages u0, v0 there and fields stages its
@@ -404,7 +426,7 @@ size_t lbs_footprint(const lbs_lattice *lat) {
   lbs_material m = {LBS_NH, 1.0, 0.3, 1.0, {0.0, 0.0}};
   Params p = make_params(lat, &m, nullptr);
   Sizes s = sizes_of(p, launchers_for(lat->precision));
-  return 2 * (s.g + s.u + s.b) + s.mon;
+  return layout_of(s).total;
 }
 
 int lbs_constitutive(int32_t model, double lam, double mu, const double H[4], double P[4], double N[4]) {
@@ -482,16 +504,29 @@ int lbs_create(const lbs_lattice *lat, const lbs_material *mat, const lbs_bcs *b
   }
   h->stream = h->own_stream;
   Sizes s = sizes_of(h->P, *h->L);
+  const Layout lay = layout_of(s);
   bool ok = true;
-  for (int i = 0; i < 2 && ok; ++i) {
-    h->g[i] = dev_alloc(h->alloc, s.g, h->stream);
-    h->u[i] = dev_alloc(h->alloc, s.u, h->stream);
-    h->b[i] = dev_alloc(h->alloc, s.b, h->stream);
-    ok = h->g[i] && h->u[i] && h->b[i];
-  }
-  if (ok) {
-    h->mon_block = dev_alloc(h->alloc, s.mon, h->stream);
-    ok = h->mon_block != nullptr;
+  h->block = dev_alloc(h->alloc, lay.total, h->stream);
+  if (h->block) {
+    char *p = (char *)h->block;
+    for (int i = 0; i < 2; ++i) {
+      h->g[i] = p + lay.g[i];
+      h->u[i] = p + lay.u[i];
+      h->b[i] = p + lay.b[i];
+    }
+    h->mon_block = p + lay.mon;
+  } else {
+    // no room for them in one piece: one by one
+    for (int i = 0; i < 2 && ok; ++i) {
+      h->g[i] = dev_alloc(h->alloc, s.g, h->stream);
+      h->u[i] = h->g[i] ? dev_alloc(h->alloc, s.u, h->stream) : nullptr;
+      h->b[i] = h->u[i] ? dev_alloc(h->alloc, s.b, h->stream) : nullptr;
+      ok = h->b[i] != nullptr;
+    }
+    if (ok) {
+      h->mon_block = dev_alloc(h->alloc, s.mon, h->stream);
+      ok = h->mon_block != nullptr;
+    }
   }
   if (ok && cudaMallocHost(&h->mon_host, 8 * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();
@@ -510,7 +545,7 @@ int lbs_create(const lbs_lattice *lat, const lbs_material *mat, const lbs_bcs *b
   }
   if (!ok) {
     lbs_destroy(h);
-    return fail(LBS_ENOMEM, "device allocation of " + std::to_string(2 * (s.g + s.u + s.b)) + " bytes failed");
+    return fail(LBS_ENOMEM, "device allocation of " + std::to_string(lay.total) + " bytes failed");
   }
   char *mb = (char *)h->mon_block;
   h->mon_partials = (double *)mb;
@@ -519,7 +554,7 @@ int lbs_create(const lbs_lattice *lat, const lbs_material *mat, const lbs_bcs *b
   h->zero_dev = h->kdev + 1;
   h->errdev = (int *)(h->kdev + 2);
   h->sev = h->kdev + 3;
-  h->bytes = 2 * (s.g + s.u + s.b) + s.mon;
+  h->bytes = lay.total;
   rc = select_variant(h, h->L->default_variant(h->P));
   // mon_out[7] holds the resident launches' barrier counters
   if (!rc && (cudaMemsetAsync(h->zero_dev, 0, 2 * sizeof(int64_t), h->stream) != cudaSuccess ||
@@ -541,12 +576,16 @@ int lbs_destroy(lbs_handle *h) {
   if (h->own_stream) cudaStreamSynchronize(h->own_stream);
   if (h->stream && h->stream != h->own_stream) cudaStreamSynchronize(h->stream);
   drop_graphs(h);
-  for (int i = 0; i < 2; ++i) {
-    dev_free(h->alloc, h->g[i], h->own_stream);
-    dev_free(h->alloc, h->u[i], h->own_stream);
-    dev_free(h->alloc, h->b[i], h->own_stream);
+  if (h->block) {
+    dev_free(h->alloc, h->block, h->own_stream);
+  } else {
+    for (int i = 0; i < 2; ++i) {
+      dev_free(h->alloc, h->g[i], h->own_stream);
+      dev_free(h->alloc, h->u[i], h->own_stream);
+      dev_free(h->alloc, h->b[i], h->own_stream);
+    }
+    dev_free(h->alloc, h->mon_block, h->own_stream);
   }
-  dev_free(h->alloc, h->mon_block, h->own_stream);
   if (h->mon_host) cudaFreeHost(h->mon_host);
   if (h->mon_event) cudaEventDestroy(h->mon_event);
   if (h->fork.side) cudaStreamSynchronize(h->fork.side);

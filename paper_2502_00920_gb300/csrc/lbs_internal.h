@@ -189,6 +189,7 @@ struct lbs_handle {
   lbs::Allocator alloc;
   cudaStream_t own_stream;
   cudaStream_t stream;
+  void *block;              // the buffers' common allocation (null: each has its own)
   void *g[2], *u[2], *b[2];
   void *mon_block;          // partials, out[8], counters
   double *mon_partials;
