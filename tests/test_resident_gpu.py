@@ -41,7 +41,7 @@ def fields(L, c, calls, **kw):
         return s.fields(), s.launch_count
 
 
-# one node more and less than the tiles (8 x 8, 16 x 8, 16 x 16, 32 x 16), the
+# one node more and less than the tiles (8 x 8, 16 x 8, 16 x 16, 32 x 14), the
 # smallest lattice, long strips, and the largest lattices on each tile
 SIZES = [(3, 3), (4, 9), (8, 8), (9, 7), (17, 8), (33, 15), (3, 300), (301, 5), (96, 96), (128, 128), (131, 125),
          (256, 256), (303, 241)]
