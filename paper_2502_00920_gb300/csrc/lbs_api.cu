@@ -672,7 +672,14 @@ int lbs_step(lbs_handle *h, int64_t n) {
       }
       rp.bar = (unsigned *)(h->mon_out + 7);
       rp.err = h->errdev;
-      LBS_CK(h->L->resident(h->P, rp, h->parity, h->k, m, h->stream));
+      const cudaError_t e = h->L->resident(h->P, rp, h->parity, h->k, m, h->stream);
+      if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+        // fewer SMs to be had than the device reports: launch every iteration
+        cudaGetLastError();
+        h->resident = false;
+        continue;
+      }
+      LBS_CK(e);
       h->launches += 1;
       h->parity ^= m & 1;
       h->k += m;
