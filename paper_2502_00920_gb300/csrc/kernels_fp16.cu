@@ -95,9 +95,9 @@ int kernels_per_step1(const Params &, int) { return 1; }
 // three side by side.  Small lattices pull from global memory (walled 300^2
 // variant 0 6.8 / 3.0, 7 11.6 / 3.6; 512^2 7.9 / 5.3, 15.4 / 5.4). Walled ones of
 // several waves take the smaller TMA tiles, which leave fewer nodes to the frame
-// tiles (4096 x 256 variant 4 22.1 / 18.6, 7 27.0 / 25.0; 1500 x 1300 38.3 / 32.5,
-// 47.3 / 36.3); the rest the larger (1021 x 509 variant 4 14.9 / 9.7, 7 16.4 / 9.5;
-// 1024^2 periodic 23.0 / 18.5, 21.6 / 17.8).
+// tiles (4096 x 256 variant 4 21.1 / 18.4, 7 24.1 / 21.3; 2650 x 463 24.4 / 20.9, 25.1
+// / 21.6; 1500 x 1300 36.6 / 31.9, 36.5 / 30.6); the rest the larger (1021 x 509
+// variant 4 15.3 / 9.9, 7 16.7 / 9.6; 1024^2 periodic 23.0 / 18.5, 21.6 / 17.8).
 int default_variant(const Params &p) {
   const int64_t nodes = (int64_t)p.nx * p.ny;
   if (nodes >= kColumnNodes) return 8;

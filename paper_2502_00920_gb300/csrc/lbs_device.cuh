@@ -1010,8 +1010,13 @@ __global__ void __launch_bounds__(C::NT) step_interior_kernel(const Params P, co
 // With SPLIT, a frame tile of CPT nodes per thread is processed as CPT
 // tiles of one node per thread by CPT blocks.  On a small lattice the frame
 // tiles are few and the iteration waits on their latency; once there are
-// more of them than SMs the pieces' extra halo work costs more than it saves
-// (launch_edge chooses).
+// many more of them than fit the SMs the pieces' extra halo work costs more
+// than it saves.  The line (launch_edge): as many tiles as SMs in FP32, twice as
+// many in FP16 storage and FP64 (us per iteration, one lattice alone / three
+// side by side, the line at once against twice the SMs: FP16 storage 4096 x 256 on
+// 32 x 16 tiles 22.6 / 18.9 -> 21.1 / 18.4, 1500 x 1300 on 32 x 32 tiles 47.8 / 36.6 ->
+// 36.5 / 30.6; FP64 4096 x 256 247 / 227 -> 242 / 225; FP32 2650 x 463 30.1 / 24.2 ->
+// 29.0 / 24.6).
 template <class C, bool SPLIT>
 struct FrameCfg {
   using type = C;
@@ -1047,7 +1052,7 @@ void launch_edge(const Params &P, const StepPtrs &S, int nedge, int ntx, int a_l
       cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
       return n > 0 ? n : 1;
     }();
-    if (nedge <= sms) {
+    if (nedge <= (sizeof(typename C::gs) == 4 ? sms : 2 * sms)) {
       using H = typename FrameCfg<C, true>::type;
       const int nb = C::CPT * nedge;
       if (P.extrap) step_edge_kernel<C, true, true><<<nb, H::NT, 0, st>>>(P, c, S, ntx, a_lo, a_hi, b_lo, b_hi);
