@@ -273,16 +273,6 @@ template <int I>
 struct Slot {
   static constexpr int value = I;
 };
-template <int T>
-constexpr int kColumnHalo = T == 1 ? 4 : 6;  // (even: pairs stay aligned)
-template <int T>
-constexpr int kColumnOut = 64 - 2 * kColumnHalo<T>;
-struct ColumnRegion {
-  int x0, x1, y0, y1;  // nodes to advance
-  int nstrip, seg;     // strips of kColumnOut columns; rows per segment
-  int wrap;            // periodic lattice: columns and rows wrap (nx even)
-};
-
 __device__ __forceinline__ void store_raw(float *p, Two a) { *reinterpret_cast<float2 *>(p) = make_float2(a.x, a.y); }
 __device__ __forceinline__ void store_raw(__half *p, uint32_t a) { *reinterpret_cast<uint32_t *>(p) = a; }
 
@@ -317,40 +307,35 @@ __global__ void __launch_bounds__(32 * T, 12 / T) step_column_kernel(const Param
   constexpr int kP = Column<Pr>::kParked > 0 ? Column<Pr>::kParked : 1;
   __shared__ Raw parked[T][2][kP][32];
   const int lane = threadIdx.x % 32, t = threadIdx.x / 32;
-  const int xo = R.x0 + (int)(blockIdx.x % R.nstrip) * kColumnOut<T>;
-  const int ya = R.y0 + (int)(blockIdx.x / R.nstrip) * R.seg, yb = min(ya + R.seg, R.y1);
-  auto row_of = [&](int r) {
-    if (R.wrap) return r < 0 ? r + P.ny : (r >= P.ny ? r - P.ny : r);
-    return min(r, P.ny - 1);
-  };
-  auto col_of = [&](int x, int last) { return R.wrap ? (x < 0 ? x + P.nx : (x >= P.nx ? x - P.nx : x)) : min(x, last); };
+  int xo, ya, yb;
+  column_block<T>(R, (int)blockIdx.x, xo, ya, yb);
   const int xc = xo - kColumnHalo<T> + 2 * lane;  // this lane's columns xc, xc + 1
-  const bool mine = 2 * lane >= kColumnHalo<T> && 2 * lane < 64 - kColumnHalo<T> && xc < R.x1;
-  const int plane = P.ny * P.pitch;
+  const bool mine = column_mine<T>(R, lane, xc);
+  const size_t plane = plane_of(P);
   // (without wrap, lanes past the last node repeat the last pair; where that
   // pair is the last node and a word of the row's padding, which holds
   // anything, the node stands for both)
-  const int xl = col_of(xc, (P.nx - 1) & ~1);
+  const int xl = column_pair(P, R, xc);
   const bool pad = xl == P.nx - 1;
   const bool pads = __any_sync(kAll, pad);
   const gs *gin = (const gs *)S.g_in + xl;
   // u is copied by whole lines: this lane brings nodes lane and lane + 32
-  const float4 *uin = (const float4 *)S.u_in + col_of(xo - kColumnHalo<T> + lane, P.nx - 1);
-  const int u32 = col_of(xo - kColumnHalo<T> + lane + 32, P.nx - 1) - col_of(xo - kColumnHalo<T> + lane, P.nx - 1);
+  const float4 *uin = (const float4 *)S.u_in + column_node(P, R, xo - kColumnHalo<T> + lane);
+  const int u32 = column_node(P, R, xo - kColumnHalo<T> + lane + 32) - column_node(P, R, xo - kColumnHalo<T> + lane);
 
   Column<Pr> col;
   col.clear();
 #pragma unroll
   for (int k = 0; k < 2 * kP; ++k) narrow(two(0.0f), parked[t][k / kP][k % kP][lane]);
-  const int r0 = ya - 3 * T, n = yb - ya + (9 * T - 3);
+  const int r0 = ya - 3 * T, n = column_steps<T>(ya, yb);
   // warp t is 5 rows behind warp t - 1 (3 that its new rows lag, 2 of the ring)
   auto fetch = [&](int j) {
     if (j < n) {
       ColumnRow<Pr> &w = rows[0][j & (kColumnRing - 1)];
-      const gs *p = gin + (size_t)row_of(r0 + j) * P.pitch;
+      const gs *p = gin + (size_t)column_row(P, R, r0 + j) * P.pitch;
 #pragma unroll
-      for (int q = 0; q < 9; ++q) copy_async<sizeof(Raw)>(&w.g[q][lane], p + (size_t)q * plane);
-      const float4 *pu = uin + (size_t)row_of(r0 + j) * P.pitch;
+      for (int q = 0; q < 9; ++q) copy_async<sizeof(Raw)>(&w.g[q][lane], p + q * plane);
+      const float4 *pu = uin + (size_t)column_row(P, R, r0 + j) * P.pitch;
       copy_async<16>(&w.u[u_slot(lane)], pu);
       copy_async<16>(&w.u[u_slot(lane + 32)], pu + u32);
     }
@@ -390,12 +375,12 @@ __global__ void __launch_bounds__(32 * T, 12 / T) step_column_kernel(const Param
       o.u[u_slot(2 * lane)] = make_float4(lo(u[0]), lo(u[1]), lo(u[2]), lo(u[3]));
       o.u[u_slot(2 * lane + 1)] = make_float4(hi(u[0]), hi(u[1]), hi(u[2]), hi(u[3]));
     } else {
-      const int row = r0 + j - 5 * (T - 1) - 3;
+      const int row = column_stored<T>(r0, j);
       if (mine && row >= ya && row < yb) {
         const size_t o = (size_t)row * P.pitch + xc;
         gs *go = (gs *)S.g_out + o;
 #pragma unroll
-        for (int q = 0; q < 9; ++q) store_raw(go + (size_t)q * plane, out[q]);
+        for (int q = 0; q < 9; ++q) store_raw(go + q * plane, out[q]);
         asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"((float4 *)S.u_out + o),
                      "f"(lo(u[0])), "f"(lo(u[1])), "f"(lo(u[2])), "f"(lo(u[3])), "f"(hi(u[0])), "f"(hi(u[1])),
                      "f"(hi(u[2])), "f"(hi(u[3]))
@@ -424,9 +409,7 @@ __global__ void __launch_bounds__(32 * T, 12 / T) step_column_kernel(const Param
   }
 }
 
-// Strips and segments of a region: the number of segments that makes the time
-// least, counted in rows marched (each segment's lead included) times rounds of
-// resident blocks (a round begun costs about half of one once there are many).
+// strips and segments of a region on this device
 template <class Pr, int T>
 ColumnRegion column_region(int x0, int x1, int y0, int y1, int wrap) {
   static const int resident = [] {
@@ -436,18 +419,7 @@ ColumnRegion column_region(int x0, int x1, int y0, int y1, int wrap) {
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, step_column_kernel<Pr, T>, 32 * T, 0);
     return (sms > 0 ? sms : 1) * (per > 0 ? per : 1);
   }();
-  ColumnRegion R{x0, x1, y0, y1, (x1 - x0 + kColumnOut<T> - 1) / kColumnOut<T>, y1 - y0, wrap};
-  int64_t best = -1;
-  for (int n = 1; n <= 512 && n * 16 <= y1 - y0 + 15; ++n) {
-    const int seg = (y1 - y0 + n - 1) / n;
-    const int64_t blocks = (int64_t)R.nstrip * ((y1 - y0 + seg - 1) / seg);
-    const int64_t cost = (blocks <= resident ? resident : blocks + resident / 2) * (seg + 9 * T - 3);
-    if (best < 0 || cost < best) {
-      best = cost;
-      R.seg = seg;
-    }
-  }
-  return R;
+  return column_split<T>(x0, x1, y0, y1, wrap, resident);
 }
 
 template <class Pr, int T>
@@ -458,12 +430,7 @@ cudaError_t launch_column(const Params &P, const StepPtrs &S, const ColumnRegion
   return cudaGetLastError();
 }
 
-// A periodic lattice goes whole through the columns (rows and columns wrap, at
-// most once; nx even, so that no lane's pair straddles the seam), T iterations
-// a launch.
-inline bool column_wraps(const Params &P) {
-  return P.per_x && P.per_y && P.nx % 2 == 0 && P.nx >= 128 && P.ny >= 64;
-}
+// a periodic lattice whole, T iterations a launch
 template <class Pr, int T>
 cudaError_t launch_column_periodic(const Params &P, const StepPtrs &S, cudaStream_t st) {
   return launch_column<Pr, T>(P, S, column_region<Pr, T>(0, P.nx, 0, P.ny, 1), st);

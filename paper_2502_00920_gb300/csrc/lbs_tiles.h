@@ -12,6 +12,7 @@
 // e.g. the kernels' Params.
 #pragma once
 #include <stddef.h>
+#include <stdint.h>
 
 #ifdef __CUDACC__
 #define LBS_HD __host__ __device__ __forceinline__
@@ -259,6 +260,92 @@ LBS_HD void edge_tile(int e, int ntx, int a_lo, int a_hi, int b_lo, int b_hi, in
   e -= mid;
   a = e % ntx;
   b = b_hi + e / ntx;
+}
+
+// ------------------------------------------------------------------ columns
+// elements of one plane of the state (past 2^31 on lattices that fit the GPU)
+template <class G>
+LBS_HD size_t plane_of(const G &P) {
+  return (size_t)P.ny * P.pitch;
+}
+
+// Warp columns: block b of the region's nstrip x segments advances the strip
+// whose first stored column is xo over the rows [ya, yb), T iterations.  A strip
+// is 64 columns, two per lane, of which kColumnHalo on each side are lost
+// (three per iteration; even, so that pairs stay aligned) and kColumnOut stored.
+template <int T>
+constexpr int kColumnHalo = T == 1 ? 4 : 6;
+template <int T>
+constexpr int kColumnOut = 64 - 2 * kColumnHalo<T>;
+struct ColumnRegion {
+  int x0, x1, y0, y1;  // nodes to advance
+  int nstrip, seg;     // strips of kColumnOut columns; rows per segment
+  int wrap;            // periodic lattice: columns and rows wrap (nx even)
+};
+LBS_HD int lower_of(int a, int b) { return a < b ? a : b; }
+template <int T>
+LBS_HD void column_block(const ColumnRegion &R, int b, int &xo, int &ya, int &yb) {
+  xo = R.x0 + (b % R.nstrip) * kColumnOut<T>;
+  ya = R.y0 + (b / R.nstrip) * R.seg;
+  yb = lower_of(ya + R.seg, R.y1);
+}
+// whether a lane stores its pair of columns xc, xc + 1
+template <int T>
+LBS_HD bool column_mine(const ColumnRegion &R, int lane, int xc) {
+  return 2 * lane >= kColumnHalo<T> && 2 * lane < 64 - kColumnHalo<T> && xc < R.x1;
+}
+// Rows fetched for a segment, from row ya - 3 T on; the row that step j stores
+// (the last warp is 5 rows behind the one before, its new rows 3 behind).
+template <int T>
+LBS_HD int column_steps(int ya, int yb) {
+  return yb - ya + (9 * T - 3);
+}
+template <int T>
+LBS_HD int column_stored(int r0, int j) {
+  return r0 + j - 5 * (T - 1) - 3;
+}
+// The row, the first column of a pair and the node that a lane reads: wrapped
+// (at most once), else held inside the lattice, where the values are unused.
+template <class G>
+LBS_HD int column_row(const G &P, const ColumnRegion &R, int r) {
+  if (R.wrap) return r < 0 ? r + P.ny : (r >= P.ny ? r - P.ny : r);
+  return lower_of(r, P.ny - 1);
+}
+template <class G>
+LBS_HD int column_at(const G &P, const ColumnRegion &R, int x, int last) {
+  return R.wrap ? (x < 0 ? x + P.nx : (x >= P.nx ? x - P.nx : x)) : lower_of(x, last);
+}
+template <class G>
+LBS_HD int column_pair(const G &P, const ColumnRegion &R, int x) {
+  return column_at(P, R, x, (P.nx - 1) & ~1);
+}
+template <class G>
+LBS_HD int column_node(const G &P, const ColumnRegion &R, int x) {
+  return column_at(P, R, x, P.nx - 1);
+}
+// A periodic lattice goes whole through the columns (rows and columns wrap, at
+// most once; nx even, so that no lane's pair straddles the seam).
+template <class G>
+LBS_HD bool column_wraps(const G &P) {
+  return P.per_x && P.per_y && P.nx % 2 == 0 && P.nx >= 128 && P.ny >= 64;
+}
+// Strips and segments of a region: the number of segments that makes the time
+// least, counted in rows marched (each segment's lead included) times rounds of
+// resident blocks (a round begun costs about half of one once there are many).
+template <int T>
+ColumnRegion column_split(int x0, int x1, int y0, int y1, int wrap, int resident) {
+  ColumnRegion R{x0, x1, y0, y1, (x1 - x0 + kColumnOut<T> - 1) / kColumnOut<T>, y1 - y0, wrap};
+  int64_t best = -1;
+  for (int n = 1; n <= 512 && n * 16 <= y1 - y0 + 15; ++n) {
+    const int seg = (y1 - y0 + n - 1) / n;
+    const int64_t blocks = (int64_t)R.nstrip * ((y1 - y0 + seg - 1) / seg);
+    const int64_t cost = (blocks <= resident ? resident : blocks + resident / 2) * (seg + 9 * T - 3);
+    if (best < 0 || cost < best) {
+      best = cost;
+      R.seg = seg;
+    }
+  }
+  return R;
 }
 
 // ------------------------------------------------------------------ TMA boxes
