@@ -96,10 +96,10 @@ __global__ void __launch_bounds__(C::NT, 3) batch_frame3_kernel(const BatchLatti
 template <class R>
 __global__ void __launch_bounds__(128) batch_edges_kernel(BatchLattice *lats, int nlats, int n) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int per = n * kEdgeEntries;
-  if (i >= (int64_t)nlats * per) return;
+  const int64_t per = (int64_t)n * kEdgeEntries;
+  if (i >= nlats * per) return;
   const BatchLattice &L = lats[i / per];
-  if (L.sev) edge_table_entry<R>(L.P, L.k, L.sev, (int)(i % per));
+  if (L.sev) edge_table_entry<R>(L.P, L.k, L.sev, i % per);
 }
 template <class R>
 cudaError_t launch_batch_edges(BatchLattice *lats, int nlats, int n, cudaStream_t st) {

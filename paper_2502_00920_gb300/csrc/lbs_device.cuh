@@ -322,9 +322,9 @@ __device__ inline void edge_entry(const Params &P, int i, int64_t k, T out[2]) {
 
 // a lattice's table of n iterations from k (one iteration every kEdgeStride bytes)
 template <class R>
-__device__ inline void edge_table_entry(const Params &P, int64_t k, void *sev, int i) {
+__device__ inline void edge_table_entry(const Params &P, int64_t k, void *sev, int64_t i) {
   char *row = (char *)sev + (size_t)(i / kEdgeEntries) * kEdgeStride;
-  const int e = i % kEdgeEntries;
+  const int e = (int)(i % kEdgeEntries);
   if (P.extrap) {
     if (e < 4) edge_entry(P, e, k + i / kEdgeEntries, ((double(*)[2])row)[e]);
   } else {

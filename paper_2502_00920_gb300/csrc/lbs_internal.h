@@ -62,10 +62,6 @@ struct StepPtrs {
                         //   edge table, device), or null: the frame tiles evaluate them
 };
 
-// Edge tables: one row of kEdgeStride bytes per iteration (edge_table_entry in
-// lbs_device.cuh); a handle keeps one of kEdgeBatch iterations.
-constexpr int kEdgeStride = 128, kEdgeBatch = 64;
-
 // Device pointers of one lattice for a resident launch: both buffers of each
 // state array, the barrier's two counters (zero between launches) and the
 // error flag.

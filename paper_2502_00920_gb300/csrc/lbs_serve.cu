@@ -85,8 +85,8 @@ struct lbs_server {
   int lat_cap = 0;
   BatchTile *d_tiles = nullptr;
   int tile_cap = 0;
-  double *d_sev = nullptr;  // the chunk's edge tables, one per lattice
-  int sev_cap = 0;
+  char *d_sev = nullptr;  // the chunk's edge tables, one per lattice
+  size_t sev_cap = 0;
   int *d_err = nullptr;
 
   double now() const { return std::chrono::duration<double>(Clock::now() - t0).count(); }
@@ -125,12 +125,12 @@ void finish(lbs_server *s, Req *r, int error) {
   s->cv_done.notify_all();
 }
 
-template <class T>
-bool ensure(T *&ptr, int &cap, int need) {
+template <class T, class N>
+bool ensure(T *&ptr, N &cap, N need) {
   if (need <= cap) return true;
   if (ptr) cudaFree(ptr);
   ptr = nullptr;
-  int c = std::max(need, 2 * cap);
+  const N c = std::max(need, 2 * cap);
   if (cudaMalloc(&ptr, sizeof(T) * (size_t)c) != cudaSuccess) {
     cudaGetLastError();
     cap = 0;
@@ -477,9 +477,14 @@ void run(lbs_server *s) {
       nl = (int)edge_lin.size();
       ht.insert(ht.end(), edge.begin(), edge.end());
       ht.insert(ht.end(), edge_lin.begin(), edge_lin.end());
-      const int sev_need = (int)hl.size() * (int)s->cfg.chunk * (lbs::kEdgeStride / 8);
-      const bool sev_ok = ensure(s->d_sev, s->sev_cap, sev_need);
-      for (size_t i = 0; i < hl.size(); ++i) hl[i].sev = sev_ok ? s->d_sev + i * (size_t)s->cfg.chunk * (lbs::kEdgeStride / 8) : nullptr;
+      // (a chunk runs no lattice past the longest one's end; without room for the
+      // tables the frame tiles evaluate the values)
+      int64_t rows = 0;
+      for (Req *r : res) rows = std::max(rows, r->nsteps - r->k);
+      rows = std::min(rows, (int64_t)s->cfg.chunk);
+      const bool sev_ok = ensure(s->d_sev, s->sev_cap, lbs::edge_tables_bytes(hl.size(), rows));
+      for (size_t i = 0; i < hl.size(); ++i)
+        hl[i].sev = sev_ok ? s->d_sev + lbs::edge_tables_bytes(i, rows) : nullptr;
       if (!ensure(s->d_lats, s->lat_cap, (int)hl.size()) || !ensure(s->d_tiles, s->tile_cap, (int)ht.size())) {
         for (Req *r : res) retire.emplace_back(r, LBS_ENOMEM);
         res.clear();

@@ -262,6 +262,19 @@ LBS_HD void edge_tile(int e, int ntx, int a_lo, int a_hi, int b_lo, int b_hi, in
   b = b_hi + e / ntx;
 }
 
+// ------------------------------------------------------------------ edge tables
+// One row of kEdgeStride bytes per iteration (edge_table_entry in
+// lbs_device.cuh); a handle keeps one of kEdgeBatch iterations.
+constexpr int kEdgeStride = 128, kEdgeBatch = 64;
+
+// Bytes of a batch's tables, one of `rows` iterations per lattice one after the
+// other; as many as never can be had where they pass 63 bits.
+LBS_HD size_t edge_tables_bytes(size_t lattices, int64_t rows) {
+  const size_t most = SIZE_MAX / 2;
+  if (lattices == 0 || rows <= 0) return 0;
+  return (size_t)rows > most / kEdgeStride / lattices ? most : lattices * (size_t)rows * kEdgeStride;
+}
+
 // ------------------------------------------------------------------ columns
 // elements of one plane of the state (past 2^31 on lattices that fit the GPU)
 template <class G>
