@@ -157,9 +157,9 @@ int lbs_set_initial_device(lbs_handle *h, const double *u0, const double *v0);
 /* Advance n >= 0 iterations (asynchronous).  Launches one fused kernel per
  * iteration, replayed from a CUDA graph in chunks (lbs_set_graph_chunk).  A
  * small lattice (up to some 68 000 nodes in single precision, 19 000 in double)
- * instead advances all n, up to the point where a monitor is due, in one
- * cooperative launch, unless lbs_set_variant chose its kernel or the graph
- * chunk is 0; the results are the same bits.
+ * instead advances all n, up to the point where a monitor is due, in
+ * cooperative launches of at most 4096 iterations, unless lbs_set_variant chose
+ * its kernel or the graph chunk is 0; the results are the same bits.
  * Returns LBS_EUNSTABLE if an earlier monitor already found a non-finite
  * value; the state then stays available for lbs_fields. */
 int lbs_step(lbs_handle *h, int64_t n);

@@ -262,7 +262,8 @@ using namespace lbs;
 
 namespace {
 
-// iterations of one resident launch at most (a few tens of milliseconds)
+// iterations of one resident launch at most (a few tens of milliseconds; times
+// its blocks, the barrier's arrivals stay far below 2^32)
 constexpr int kResidentMost = 4096;
 
 // row: the iteration's row of the handle's edge table, -1: the frame tiles
@@ -655,15 +656,19 @@ int lbs_step(lbs_handle *h, int64_t n) {
   int rc = check_monitor(h, false);
   if (rc) return rc;
   int64_t table_from = 0, table_end = 0;  // iterations the edge table holds
+  int64_t run = 0;                        // what is left up to a resident run's boundary
   while (n > 0) {
     if (h->resident && h->graph_chunk > 0) {
       // the iterations up to the end or the point where a monitor is due: the
       // first boundary at or after it of the graph chunks (and of the single
-      // iterations that follow them)
-      int m = 0;
-      do {
-        m += n - m >= h->graph_chunk ? h->graph_chunk : 1;
-      } while (m < n && m < kResidentMost && !(h->mon_interval > 0 && h->k + m >= h->next_mon));
+      // iterations that follow them); a chunk of any length goes out in
+      // launches of kResidentMost
+      if (run == 0) {
+        do {
+          run += n - run >= h->graph_chunk ? h->graph_chunk : 1;
+        } while (run < n && run < kResidentMost && !(h->mon_interval > 0 && h->k + run >= h->next_mon));
+      }
+      const int m = (int)std::min<int64_t>(run, kResidentMost);
       ResidentPtrs rp;
       for (int i = 0; i < 2; ++i) {
         rp.g[i] = h->g[i];
@@ -677,6 +682,7 @@ int lbs_step(lbs_handle *h, int64_t n) {
         // fewer SMs to be had than the device reports: launch every iteration
         cudaGetLastError();
         h->resident = false;
+        run = 0;
         continue;
       }
       LBS_CK(e);
@@ -684,6 +690,8 @@ int lbs_step(lbs_handle *h, int64_t n) {
       h->parity ^= m & 1;
       h->k += m;
       n -= m;
+      run -= m;
+      if (run > 0) continue;
     } else if (h->graph_chunk > 0 && n >= h->graph_chunk) {
       if (!h->graph[h->parity] || h->graph_variant[h->parity] != h->variant) {
         if (h->graph[h->parity]) {
