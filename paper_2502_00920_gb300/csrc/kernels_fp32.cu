@@ -151,9 +151,10 @@ void coef(const Params &p, void *out) {
 using RS = ResCfg<P, 16, 8>;
 using RL = ResCfg<P, 32, 14>;
 int resident_large(const Params &p) { return p.extrap ? resident_sms() / 2 : resident_sms(); }
-bool resident_applies(const Params &p) { return resident_shape<RS, RL>(p, resident_large(p)) != kResidentNone; }
-cudaError_t resident(const Params &p, const ResidentPtrs &s, int parity, int64_t k0, int n, cudaStream_t st) {
-  return launch_resident<RS, RL>(p, s, parity, k0, n, resident_large(p), st);
+int resident_plan(const Params &p) { return choose_resident<RS, RL>(p, resident_large(p)); }
+cudaError_t resident(const Params &p, const ResidentPtrs &s, int plan, int parity, int64_t k0, int n,
+                     cudaStream_t st) {
+  return launch_resident<RS, RL>(p, s, plan, parity, k0, n, st);
 }
 
 // the server's batch tile shapes: the global-memory tiles V0-V3
@@ -183,7 +184,7 @@ const Launchers kL = {kVariants,
                       launch_edge_table<P::real>,
                       launch_batch_edges<P::real>,
                       coef,
-                      resident_applies,
+                      resident_plan,
                       resident,
                       tma_maps,
                       launch_init<V0>,

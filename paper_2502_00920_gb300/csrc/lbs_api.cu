@@ -561,7 +561,7 @@ int lbs_create(const lbs_lattice *lat, const lbs_material *mat, const lbs_bcs *b
   if (!rc && (cudaMemsetAsync(h->zero_dev, 0, 2 * sizeof(int64_t), h->stream) != cudaSuccess ||
               cudaMemsetAsync(h->mon_out + 7, 0, sizeof(double), h->stream) != cudaSuccess))
     rc = LBS_ECUDA;
-  h->resident = h->L->resident_applies(h->P);
+  h->resident = h->L->resident_plan(h->P);
   if (!rc) rc = lbs_set_initial_device(h, nullptr, nullptr);
   if (!rc && cudaStreamSynchronize(h->stream) != cudaSuccess) rc = fail(LBS_ECUDA, "initialisation failed");
   if (rc) {
@@ -677,11 +677,18 @@ int lbs_step(lbs_handle *h, int64_t n) {
       }
       rp.bar = (unsigned *)(h->mon_out + 7);
       rp.err = h->errdev;
-      const cudaError_t e = h->L->resident(h->P, rp, h->parity, h->k, m, h->stream);
+      const cudaError_t e = h->L->resident(h->P, rp, h->resident, h->parity, h->k, m, h->stream);
+      if (e != cudaSuccess && h->resident == kResidentCluster) {
+        // the cluster is refused: the grid barrier instead (which reports what
+        // else may be wrong)
+        cudaGetLastError();
+        h->resident = kResidentSmall;
+        continue;
+      }
       if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
         // fewer SMs to be had than the device reports: launch every iteration
         cudaGetLastError();
-        h->resident = false;
+        h->resident = kResidentNone;
         run = 0;
         continue;
       }
@@ -901,7 +908,7 @@ int lbs_set_variant(lbs_handle *h, int32_t variant) {
   if (!h || variant < 0 || variant >= h->L->nvariants) return fail(LBS_EINVAL, "unknown tile variant");
   if (variant != h->variant) LBS_CK(cudaStreamSynchronize(h->stream));
   const int rc = select_variant(h, variant);
-  if (!rc) h->resident = false;  // the caller's choice of step kernel
+  if (!rc) h->resident = kResidentNone;  // the caller's choice of step kernel
   return rc;
 }
 
@@ -913,7 +920,7 @@ int lbs_autotune_handle(lbs_handle *h, int32_t steps) {
   rc = lbs_set_variant(h, best);
   // the variants are what single launches run on; a small lattice's longer
   // runs stay resident
-  if (!rc) h->resident = h->L->resident_applies(h->P);
+  if (!rc) h->resident = h->L->resident_plan(h->P);
   return rc;
 }
 

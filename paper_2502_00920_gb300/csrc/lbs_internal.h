@@ -62,6 +62,10 @@ struct StepPtrs {
                         //   edge table, device), or null: the frame tiles evaluate them
 };
 
+// How a lattice's resident launches run: not at all, on small tiles behind a
+// grid barrier, the same as one thread-block cluster, on large tiles.
+enum { kResidentNone = 0, kResidentSmall = 1, kResidentCluster = 2, kResidentLarge = 3 };
+
 // Device pointers of one lattice for a resident launch: both buffers of each
 // state array, the barrier's two counters (zero between launches) and the
 // error flag.
@@ -126,9 +130,11 @@ struct Launchers {
   // a batch's table (out: 32 doubles of room)
   void (*coef)(const Params &p, void *out);
   // n iterations in one cooperative launch, for the lattices where that is
-  // faster than launching every iteration (resident_applies)
-  bool (*resident_applies)(const Params &p);
-  cudaError_t (*resident)(const Params &p, const ResidentPtrs &s, int parity, int64_t k0, int n, cudaStream_t st);
+  // faster than launching every iteration (resident_plan on the current device,
+  // one of kResident*)
+  int (*resident_plan)(const Params &p);
+  cudaError_t (*resident)(const Params &p, const ResidentPtrs &s, int plan, int parity, int64_t k0, int n,
+                          cudaStream_t st);
   // TMA descriptors of one (g, u) buffer pair for a tile variant; returns
   // false if the variant does not use TMA.  out_g/out_u: CUtensorMap storage.
   bool (*tma_maps)(const Params &p, int variant, const void *g, const void *u, void *out_g, void *out_u);
@@ -202,7 +208,7 @@ struct lbs_handle {
   int64_t kdev_value;       // value held by *kdev (host mirror)
   int64_t unstable_at;
   int graph_chunk;
-  bool resident;            // runs of graph_chunk > 0 go out as resident launches
+  int resident;             // kResident*: runs of graph_chunk > 0 go out as resident launches
   cudaGraphExec_t graph[2];
   int graph_variant[2];
   size_t bytes;

@@ -2,6 +2,8 @@
 // cooperative launch.  Included by kernels_fp64.cu / kernels_fp32.cu /
 // kernels_fp16.cu after lbs_device.cuh.
 #pragma once
+#include <atomic>
+
 #include "lbs_device.cuh"
 
 namespace lbs {
@@ -236,27 +238,44 @@ __global__ void __launch_bounds__(C::NT) resident_kernel(const Params P, const C
   }
 }
 
+// A figure of the current device, evaluated once per device.
+class PerDevice {
+ public:
+  template <class F>
+  int get(F f) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return f(dev);
+    int x = v_[dev].load(std::memory_order_relaxed);
+    if (x == 0) {
+      x = f(dev) + 1;
+      v_[dev].store(x, std::memory_order_relaxed);
+    }
+    return x - 1;
+  }
+
+ private:
+  static constexpr int kDevices = 64;
+  std::atomic<int> v_[kDevices] = {};  // the figure plus one, 0: not evaluated yet
+};
+
+inline int resident_sms() {
+  static PerDevice sms;
+  return sms.get([](int dev) {
+    int n = 0;
+    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+    return n;
+  });
+}
+
 // blocks of a resident kernel that are on the GPU at once
 template <class C, bool LIN>
 int resident_capacity() {
-  static const int cap = [] {
-    int dev = 0, sms = 0, per = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, resident_kernel<C, LIN, false>, C::NT, 0);
-    return sms * per;
-  }();
-  return cap;
-}
-
-inline int resident_sms() {
-  static const int sms = [] {
-    int dev = 0, n = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+  static PerDevice per;
+  return resident_sms() * per.get([](int) {
+    int n = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, resident_kernel<C, LIN, false>, C::NT, 0);
     return n;
-  }();
-  return sms;
+  });
 }
 
 template <class C>
@@ -265,34 +284,20 @@ int resident_tiles(const Params &P) {
   return n < (1 << 20) ? (int)n : 1 << 20;
 }
 
-// The tile a lattice's resident launches run on: the small one while every
-// tile has an SM of its own, the large one while its tiles number at most
-// `large_most`, none (0) for larger lattices, which advance one iteration per
-// launch.  Small tiles have the shorter iteration, large ones reach further
-// and leave room for other lattices' launches (each shape's lines are
-// measured at the precisions' instantiations).
-enum { kResidentNone = 0, kResidentSmall = 1, kResidentLarge = 2 };
-template <class Small, class Large>
-int resident_shape(const Params &P, int large_most) {
-  const int cs = P.extrap ? resident_capacity<Small, true>() : resident_capacity<Small, false>();
-  const int cl = P.extrap ? resident_capacity<Large, true>() : resident_capacity<Large, false>();
-  const int ns = resident_tiles<Small>(P), nl = resident_tiles<Large>(P);
-  if (ns <= resident_sms() && ns <= cs) return kResidentSmall;
-  if (nl <= large_most && nl <= cl) return kResidentLarge;
-  return kResidentNone;
-}
-
-// largest cluster of resident blocks: 16 (non-portable) where the GPU places
-// one, else 0
+// Largest cluster of resident blocks: 16 (non-portable) where the GPU places
+// one, else 0.  The permission belongs to the kernel on one device (and ends
+// with its context), so it is given for every handle; a launch without it is
+// refused.
 constexpr int kClusterMost = 16;
 template <class C, bool LIN>
 int resident_cluster() {
-  static const int most = [] {
-    if (cudaFuncSetAttribute(resident_kernel<C, LIN, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
-        cudaSuccess) {
-      cudaGetLastError();
-      return 0;
-    }
+  if (cudaFuncSetAttribute(resident_kernel<C, LIN, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
+      cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  static PerDevice most;
+  return most.get([](int) {
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute at[1];
     cfg.gridDim = dim3(kClusterMost);
@@ -307,8 +312,28 @@ int resident_cluster() {
       n = 0;
     }
     return n > 0 ? kClusterMost : 0;
-  }();
-  return most;
+  });
+}
+
+// How a lattice's resident launches run, chosen once per handle on its device:
+// on the small tile while every tile has an SM of its own (as one cluster where
+// that holds them), on the large one while its tiles number at most
+// `large_most`, not at all (kResidentNone) for larger lattices, which advance
+// one iteration per launch.  Small tiles have the shorter iteration, large ones
+// reach further and leave room for other lattices' launches (each shape's lines
+// are measured at the precisions' instantiations).
+template <class Small, class Large, bool LIN>
+int choose_resident_of(const Params &P, int large_most) {
+  const int ns = resident_tiles<Small>(P), nl = resident_tiles<Large>(P);
+  if (ns <= resident_sms() && ns <= resident_capacity<Small, LIN>())
+    return ns > 1 && ns <= kClusterMost && ns <= resident_cluster<Small, LIN>() ? kResidentCluster : kResidentSmall;
+  if (nl <= large_most && nl <= resident_capacity<Large, LIN>()) return kResidentLarge;
+  return kResidentNone;
+}
+template <class Small, class Large>
+int choose_resident(const Params &P, int large_most) {
+  return P.extrap ? choose_resident_of<Small, Large, true>(P, large_most)
+                  : choose_resident_of<Small, Large, false>(P, large_most);
 }
 
 template <class C, bool LIN>
@@ -329,11 +354,12 @@ cudaError_t launch_resident_cluster(const Params &P, const ResidentPtrs &S, int 
 
 // (only the small tile has lattices of so few)
 template <class C, bool SMALL>
-cudaError_t launch_resident_c(const Params &P, const ResidentPtrs &S, int parity, int64_t k0, int n, cudaStream_t st) {
+cudaError_t launch_resident_c(const Params &P, const ResidentPtrs &S, bool cluster, int parity, int64_t k0, int n,
+                              cudaStream_t st) {
   int ntx = (P.nx + C::TX - 1) / C::TX, nty = (P.ny + C::TY - 1) / C::TY;
   const int ntiles = ntx * nty;
   if constexpr (SMALL) {
-    if (ntiles > 1 && ntiles <= (P.extrap ? resident_cluster<C, true>() : resident_cluster<C, false>()))
+    if (cluster)
       return P.extrap ? launch_resident_cluster<C, true>(P, S, parity, k0, n, ntx, ntiles, st)
                       : launch_resident_cluster<C, false>(P, S, parity, k0, n, ntx, ntiles, st);
   }
@@ -345,11 +371,12 @@ cudaError_t launch_resident_c(const Params &P, const ResidentPtrs &S, int parity
 }
 
 template <class Small, class Large>
-cudaError_t launch_resident(const Params &P, const ResidentPtrs &S, int parity, int64_t k0, int n, int large_most,
+cudaError_t launch_resident(const Params &P, const ResidentPtrs &S, int plan, int parity, int64_t k0, int n,
                             cudaStream_t st) {
-  switch (resident_shape<Small, Large>(P, large_most)) {
-    case kResidentSmall: return launch_resident_c<Small, true>(P, S, parity, k0, n, st);
-    case kResidentLarge: return launch_resident_c<Large, false>(P, S, parity, k0, n, st);
+  switch (plan) {
+    case kResidentSmall:
+    case kResidentCluster: return launch_resident_c<Small, true>(P, S, plan == kResidentCluster, parity, k0, n, st);
+    case kResidentLarge: return launch_resident_c<Large, false>(P, S, false, parity, k0, n, st);
     default: return cudaErrorInvalidValue;
   }
 }
