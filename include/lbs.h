@@ -161,13 +161,17 @@ int lbs_set_initial_device(lbs_handle *h, const double *u0, const double *v0);
  * cooperative launches of at most 4096 iterations, unless lbs_set_variant chose
  * its kernel or the graph chunk is 0; the results are the same bits.
  * Returns LBS_EUNSTABLE if an earlier monitor already found a non-finite
- * value; the state then stays available for lbs_fields. */
+ * value; the state then stays available for lbs_fields.  Returns LBS_ETIMEOUT
+ * if an earlier call found that a kernel had given up (lbs_sync). */
 int lbs_step(lbs_handle *h, int64_t n);
 
 /* Wait for the handle's work; LBS_EUNSTABLE if a monitor found a
  * non-finite value (lbs_unstable_iteration tells where), LBS_ETIMEOUT if a
  * kernel gave up waiting for its tile copies or for its other blocks (bounded
- * wait; the state is then not advanced for the affected tiles). */
+ * wait).  The state is then not advanced everywhere: every call that waits for
+ * the handle's work and reads its state (lbs_fields, lbs_fields_static,
+ * lbs_probe, lbs_monitor, lbs_grid_error, lbs_save) returns LBS_ETIMEOUT too,
+ * until lbs_set_initial or lbs_load sets the state anew. */
 int lbs_sync(lbs_handle *h);
 
 /* Fields at the current iteration into caller-owned HOST buffers (any may be
@@ -279,6 +283,14 @@ int lbs_load(lbs_handle *h, const void *buf, size_t bytes);
  * Synchronous; allocates a 4-byte flag.  Errors: LBS_EINVAL (tx_bytes >=
  * 2^20, polls == 0, timed_out NULL), LBS_ECUDA. */
 int lbs_selftest_bounded_wait(uint32_t tx_bytes, uint32_t polls, int32_t *timed_out, double *seconds);
+
+/* The same for the barrier between the blocks of a resident launch (lbs_step):
+ * launches the handle's next two iterations with one arrival taken from the
+ * barrier's count, so that every block gives up after `polls` polls and
+ * returns.  Asynchronous: the handle reports LBS_ETIMEOUT (lbs_sync) and takes
+ * a new state like any other.  Errors: LBS_EINVAL (polls == 0, or a lattice
+ * whose launches have no such barrier), LBS_ECUDA. */
+int lbs_selftest_resident_wait(lbs_handle *h, uint32_t polls);
 
 /* The handle's current tile variant (LBS_EINVAL for a null handle). */
 int32_t lbs_variant(const lbs_handle *h);

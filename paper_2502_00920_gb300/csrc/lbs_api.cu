@@ -253,6 +253,26 @@ static double *scratch_take(Scratch &s, size_t bytes) {
 
 __global__ void set_counter_kernel(int64_t *k, int64_t v) { *k = v; }
 __global__ void add_counter_kernel(int64_t *k, int64_t d) { *k += d; }
+// A state set anew: iteration 0, no monitor, the resident launches' barrier at
+// zero and no wait given up (a launch that gave up leaves its arrivals counted).
+__global__ void reset_state_kernel(int64_t *k, double *mon_out, int *err) {
+  *k = 0;
+  for (int i = 0; i < 8; ++i) mon_out[i] = 0.0;
+  *err = 0;
+}
+
+cudaError_t queue_flag(lbs_handle *h) {
+  return cudaMemcpyAsync(h->mon_host + 7, h->errdev, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+}
+int check_flag(lbs_handle *h) {
+  int gave_up;
+  memcpy(&gave_up, h->mon_host + 7, sizeof(int));
+  if (gave_up) h->gave_up = true;
+  if (!h->gave_up) return LBS_OK;
+  set_error("a kernel gave up waiting for its tile copies or its other blocks: the state is not advanced "
+            "everywhere; set it anew");
+  return LBS_ETIMEOUT;
+}
 
 }  // namespace lbs
 
@@ -283,6 +303,20 @@ StepPtrs ptrs(const lbs_handle *h, int parity, const int64_t *kptr, int64_t koff
   s.err = h->errdev;
   s.fork = h->fork.side ? &h->fork : nullptr;
   s.sev = row >= 0 ? (const char *)h->sev + (size_t)row * kEdgeStride : nullptr;
+  return s;
+}
+
+// (mon_out[7] holds the barrier's counters)
+ResidentPtrs resident_ptrs(const lbs_handle *h, uint32_t polls) {
+  ResidentPtrs s;
+  for (int i = 0; i < 2; ++i) {
+    s.g[i] = h->g[i];
+    s.u[i] = h->u[i];
+    s.b[i] = h->b[i];
+  }
+  s.bar = (unsigned *)(h->mon_out + 7);
+  s.err = h->errdev;
+  s.polls = polls;
   return s;
 }
 
@@ -333,12 +367,15 @@ int capture_graph(lbs_handle *h, int parity) {
 
 // read back a finished monitor; returns LBS_EUNSTABLE once a non-finite value was seen
 int check_monitor(lbs_handle *h, bool wait) {
+  if (h->gave_up) return check_flag(h);
   if (h->unstable_at >= 0) return LBS_EUNSTABLE;
   if (!h->mon_pending) return LBS_OK;
   cudaError_t q = wait ? cudaEventSynchronize(h->mon_event) : cudaEventQuery(h->mon_event);
   if (q == cudaErrorNotReady) return LBS_OK;
   LBS_CK(q);
   h->mon_pending = false;
+  const int rc = check_flag(h);
+  if (rc) return rc;
   if (h->mon_host[5] != 0.0) {
     h->unstable_at = (int64_t)h->mon_host[6];
     return fail(LBS_EUNSTABLE, "non-finite value at iteration " + std::to_string(h->unstable_at));
@@ -350,6 +387,7 @@ int launch_monitor_async(lbs_handle *h) {
   LBS_CK(h->L->monitor(h->P, h->g[h->parity], h->u[h->parity], h->mon_partials, monitor_blocks(h->P), h->mon_out,
                        h->k, h->stream));
   LBS_CK(cudaMemcpyAsync(h->mon_host, h->mon_out, 7 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+  LBS_CK(queue_flag(h));
   LBS_CK(cudaEventRecord(h->mon_event, h->stream));
   h->launches += 2;
   h->mon_pending = true;
@@ -374,11 +412,11 @@ int reset_state_counters(lbs_handle *h) {
   h->unstable_at = -1;
   h->mon_pending = false;
   h->next_mon = h->mon_interval;
-  set_counter_kernel<<<1, 1, 0, h->stream>>>(h->kdev, 0);
+  reset_state_kernel<<<1, 1, 0, h->stream>>>(h->kdev, h->mon_out, h->errdev);
   LBS_CK(cudaGetLastError());
   h->launches += 1;
   h->kdev_value = 0;
-  LBS_CK(cudaMemsetAsync(h->mon_out, 0, 7 * sizeof(double), h->stream));
+  h->gave_up = false;
   return LBS_OK;
 }
 
@@ -557,10 +595,7 @@ int lbs_create(const lbs_lattice *lat, const lbs_material *mat, const lbs_bcs *b
   h->sev = h->kdev + 3;
   h->bytes = lay.total;
   rc = select_variant(h, h->L->default_variant(h->P));
-  // mon_out[7] holds the resident launches' barrier counters
-  if (!rc && (cudaMemsetAsync(h->zero_dev, 0, 2 * sizeof(int64_t), h->stream) != cudaSuccess ||
-              cudaMemsetAsync(h->mon_out + 7, 0, sizeof(double), h->stream) != cudaSuccess))
-    rc = LBS_ECUDA;
+  if (!rc && cudaMemsetAsync(h->zero_dev, 0, 2 * sizeof(int64_t), h->stream) != cudaSuccess) rc = LBS_ECUDA;
   h->resident = h->L->resident_plan(h->P);
   if (!rc) rc = lbs_set_initial_device(h, nullptr, nullptr);
   if (!rc && cudaStreamSynchronize(h->stream) != cudaSuccess) rc = fail(LBS_ECUDA, "initialisation failed");
@@ -669,15 +704,7 @@ int lbs_step(lbs_handle *h, int64_t n) {
         } while (run < n && run < kResidentMost && !(h->mon_interval > 0 && h->k + run >= h->next_mon));
       }
       const int m = (int)std::min<int64_t>(run, kResidentMost);
-      ResidentPtrs rp;
-      for (int i = 0; i < 2; ++i) {
-        rp.g[i] = h->g[i];
-        rp.u[i] = h->u[i];
-        rp.b[i] = h->b[i];
-      }
-      rp.bar = (unsigned *)(h->mon_out + 7);
-      rp.err = h->errdev;
-      const cudaError_t e = h->L->resident(h->P, rp, h->resident, h->parity, h->k, m, h->stream);
+      const cudaError_t e = h->L->resident(h->P, resident_ptrs(h, kMaxBarrierPolls), h->resident, h->parity, h->k, m, h->stream);
       if (e != cudaSuccess && h->resident == kResidentCluster) {
         // the cluster is refused: the grid barrier instead (which reports what
         // else may be wrong)
@@ -764,11 +791,23 @@ int lbs_step(lbs_handle *h, int64_t n) {
 
 int lbs_sync(lbs_handle *h) {
   if (!h) return fail(LBS_EINVAL, "null handle");
+  LBS_CK(queue_flag(h));
   LBS_CK(cudaStreamSynchronize(h->stream));
-  int err = 0;
-  LBS_CK(cudaMemcpy(&err, h->errdev, sizeof(int), cudaMemcpyDeviceToHost));
-  if (err) return fail(LBS_ETIMEOUT, "a kernel gave up waiting for its tile copies");
-  return check_monitor(h, true);
+  const int rc = check_flag(h);
+  return rc ? rc : check_monitor(h, true);
+}
+
+int lbs_selftest_resident_wait(lbs_handle *h, uint32_t polls) {
+  if (!h || polls == 0) return fail(LBS_EINVAL, "bad self-test arguments");
+  if (h->resident != kResidentSmall && h->resident != kResidentLarge)
+    return fail(LBS_EINVAL, "no grid barrier in this lattice's launches");
+  // one arrival too few: the count starts at -1, and two iterations of a grid
+  // of at least two blocks wait for all of them once
+  LBS_CK(cudaMemsetAsync(h->mon_out + 7, 0xff, sizeof(unsigned), h->stream));
+  LBS_CK(h->L->resident(h->P, resident_ptrs(h, polls), h->resident, h->parity, h->k, 2, h->stream));
+  h->launches += 1;
+  h->k += 2;
+  return LBS_OK;
 }
 
 int lbs_fields_device(lbs_handle *h, double *u, double *v, double *P) {
@@ -811,7 +850,9 @@ int lbs_fields(lbs_handle *h, double *u, double *v, double *P) {
       done[i] = true;
     }
   }
+  if (!rc && queue_flag(h) != cudaSuccess) rc = fail(LBS_ECUDA, "field output failed");
   if (cudaStreamSynchronize(h->stream) != cudaSuccess && !rc) rc = fail(LBS_ECUDA, "field output failed");
+  if (!rc) rc = check_flag(h);
   for (int i = 0; i < 3; ++i) dev_free(h->alloc, owned[i], h->stream);
   return rc;
 }
@@ -830,8 +871,9 @@ int lbs_probe(lbs_handle *h, int32_t n, const int32_t *idx, double *out) {
   if (cudaMemcpyAsync(didx, idx, n * sizeof(int32_t), cudaMemcpyHostToDevice, h->stream) != cudaSuccess ||
       h->L->probe(h->P, h->u[h->parity], didx, n, dout, h->stream) != cudaSuccess ||
       cudaMemcpyAsync(out, dout, (size_t)n * 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||
-      cudaStreamSynchronize(h->stream) != cudaSuccess)
+      queue_flag(h) != cudaSuccess || cudaStreamSynchronize(h->stream) != cudaSuccess)
     rc = fail(LBS_ECUDA, "probe failed");
+  if (!rc) rc = check_flag(h);
   h->launches += 1;
   dev_free(h->alloc, buf, h->stream);
   return rc;
@@ -845,10 +887,11 @@ int lbs_grid_error_device(lbs_handle *h, const double *u_ref, double out[2]) {
   h->launches += 2;
   double o[3];
   LBS_CK(cudaMemcpyAsync(o, h->mon_out, 3 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+  LBS_CK(queue_flag(h));
   LBS_CK(cudaStreamSynchronize(h->stream));
   out[0] = o[0];
   out[1] = o[1];
-  return LBS_OK;
+  return check_flag(h);
 }
 
 int lbs_grid_error(lbs_handle *h, const double *u_ref, double out[2]) {
@@ -884,7 +927,7 @@ int lbs_monitor(lbs_handle *h, lbs_monitors *out) {
   out->momentum[1] = h->mon_host[3];
   out->mass = h->mon_host[4];
   if (h->mon_host[5] != 0.0 && h->unstable_at < 0) h->unstable_at = (int64_t)h->mon_host[6];
-  return LBS_OK;
+  return check_flag(h);
 }
 
 int lbs_set_monitor_interval(lbs_handle *h, int64_t m) {
@@ -990,8 +1033,11 @@ int lbs_load(lbs_handle *h, const void *buf, size_t bytes) {
   h->unstable_at = -1;
   h->mon_pending = false;
   h->next_mon = h->mon_interval > 0 ? (h->k / h->mon_interval + 1) * h->mon_interval : 0;
-  LBS_CK(cudaMemsetAsync(h->mon_out, 0, 7 * sizeof(double), h->stream));
+  // (as reset_state_kernel: mon_out with the barrier's counters, the flag)
+  LBS_CK(cudaMemsetAsync(h->mon_out, 0, 8 * sizeof(double), h->stream));
+  LBS_CK(cudaMemsetAsync(h->errdev, 0, sizeof(int), h->stream));
   LBS_CK(cudaStreamSynchronize(h->stream));
+  h->gave_up = false;
   return LBS_OK;
 }
 

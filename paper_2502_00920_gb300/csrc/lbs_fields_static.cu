@@ -169,9 +169,10 @@ extern "C" int lbs_fields_static(lbs_handle *h, double *u, double *v, double *P)
                               h->stream) != cudaSuccess))
       return fail_queued("lbs_fields_static: copy to host failed");
   }
+  if ((e = queue_flag(h)) != cudaSuccess) return fail_queued(std::string("lbs_fields_static: ") + cudaGetErrorString(e));
   if ((e = cudaStreamSynchronize(h->stream)) != cudaSuccess) {
     set_error(std::string("lbs_fields_static: ") + cudaGetErrorString(e));
     return LBS_ECUDA;
   }
-  return LBS_OK;
+  return check_flag(h);
 }

@@ -62,9 +62,13 @@ struct StepPtrs {
                         //   edge table, device), or null: the frame tiles evaluate them
 };
 
-// How a lattice's resident launches run: not at all, on small tiles behind a
-// grid barrier, the same as one thread-block cluster, on large tiles.
-enum { kResidentNone = 0, kResidentSmall = 1, kResidentCluster = 2, kResidentLarge = 3 };
+// How a lattice's resident launches run: not at all, on one small tile, on small
+// tiles behind a grid barrier or as one thread-block cluster, on large tiles
+// behind a grid barrier.
+enum { kResidentNone = 0, kResidentOne, kResidentSmall, kResidentCluster, kResidentLarge };
+
+// polls of a resident launch's barrier at most (seconds)
+constexpr uint32_t kMaxBarrierPolls = 1u << 22;
 
 // Device pointers of one lattice for a resident launch: both buffers of each
 // state array, the barrier's two counters (zero between launches) and the
@@ -73,6 +77,7 @@ struct ResidentPtrs {
   void *g[2], *u[2], *b[2];
   unsigned *bar;
   int *err;
+  uint32_t polls;  // of the barrier, after which a block gives up
 };
 
 struct TileShape {
@@ -198,7 +203,7 @@ struct lbs_handle {
   double *mon_out;          // device: bad, max|u|, mx, my, mass, flag
   int64_t *kdev;            // device iteration base used by graph replays
   int64_t *zero_dev;        // device constant 0 (direct launches)
-  double *mon_host;         // pinned copy of mon_out
+  double *mon_host;         // pinned copy of mon_out's first seven, then of the flag
   cudaEvent_t mon_event;
   bool mon_pending;
   int64_t mon_k;            // iteration of the pending monitor
@@ -216,6 +221,7 @@ struct lbs_handle {
   int64_t launches;         // kernels launched for this handle
   void *sev;                // edge table of kEdgeBatch iterations
   int *errdev;              // device flag: a bounded wait in a kernel gave up
+  bool gave_up;             // the flag was seen set (until the state is set anew)
   CUtensorMap tm_g[2];      // TMA descriptors of g[0], g[1] and u[0], u[1]
   CUtensorMap tm_u[2];      //   for the current variant (TMA variants only)
   bool tma;                 // the current variant stages tiles with TMA
@@ -224,3 +230,13 @@ struct lbs_handle {
   lbs_material mat;
   lbs_bcs bcs;
 };
+
+namespace lbs {
+
+// The flag of a wait given up: queue a copy of it to the host on the handle's
+// stream; once that has been waited for, LBS_ETIMEOUT (with its message) if it
+// is set or was seen set since the state was set.
+cudaError_t queue_flag(lbs_handle *h);
+int check_flag(lbs_handle *h);
+
+}  // namespace lbs

@@ -24,18 +24,17 @@ struct ResCfg {
 };
 
 // Barrier over the blocks of one cooperative launch: every block adds one to
-// *count, thread 0 polls until `target` arrivals (a bounded number of times:
-// false, with *err set, if they do not come).  The release of the arrival
+// *count, thread 0 polls until `target` arrivals (at most `polls` times: false,
+// with *err set, if they do not come).  The release of the arrival
 // covers the block's stores (ordered before it by the block barrier), the
 // acquire of the poll the reads that follow.
-constexpr uint32_t kMaxBarrierPolls = 1u << 22;
-__device__ __forceinline__ bool grid_barrier(unsigned *count, unsigned target, int *err) {
+__device__ __forceinline__ bool grid_barrier(unsigned *count, unsigned target, uint32_t polls, int *err) {
   __syncthreads();
   int ok = 1;
   if (threadIdx.x == 0) {
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
     ok = 0;
-    for (uint32_t i = 0; i < kMaxBarrierPolls; ++i) {
+    for (uint32_t i = 0; i < polls; ++i) {
       unsigned v;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(count) : "memory");
       if (v >= target) {
@@ -60,7 +59,9 @@ constexpr int kSevBatch = 32;
 // it, so it never travels), and own nodes keep their g.  g and the walls' N go
 // through L2, both buffers in turn; u is stored by the last iteration.  The
 // barrier's counters are zero between launches: the last block to leave clears
-// them.  A launch that finds the error flag set does nothing.
+// them.  Where a block gives up waiting, the counters stay as they are and the
+// error flag is set; a launch that finds it set does nothing, until setting the
+// state anew clears both.
 // What bounds an iteration: latency. Of the 2.9 us on a 16 x 8 FP32 tile the
 // grid barrier takes 1.0, the loads from L2 0.4, the three phases the rest (FP64:
 // its operations' own latency, some 300 cycles each in chains of about 35).
@@ -226,7 +227,7 @@ __global__ void __launch_bounds__(C::NT) resident_kernel(const Params P, const C
     if (CLUSTER) {
       asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     } else if (it + 1 < n && gridDim.x > 1) {
-      if (!grid_barrier(S.bar, (unsigned)(it + 1) * gridDim.x, S.err)) return;
+      if (!grid_barrier(S.bar, (unsigned)(it + 1) * gridDim.x, S.polls, S.err)) return;
     } else {
       __syncthreads();
     }
@@ -325,8 +326,10 @@ int resident_cluster() {
 template <class Small, class Large, bool LIN>
 int choose_resident_of(const Params &P, int large_most) {
   const int ns = resident_tiles<Small>(P), nl = resident_tiles<Large>(P);
-  if (ns <= resident_sms() && ns <= resident_capacity<Small, LIN>())
-    return ns > 1 && ns <= kClusterMost && ns <= resident_cluster<Small, LIN>() ? kResidentCluster : kResidentSmall;
+  if (ns <= resident_sms() && ns <= resident_capacity<Small, LIN>()) {
+    if (ns == 1) return kResidentOne;
+    return ns <= kClusterMost && ns <= resident_cluster<Small, LIN>() ? kResidentCluster : kResidentSmall;
+  }
   if (nl <= large_most && nl <= resident_capacity<Large, LIN>()) return kResidentLarge;
   return kResidentNone;
 }
@@ -374,6 +377,7 @@ template <class Small, class Large>
 cudaError_t launch_resident(const Params &P, const ResidentPtrs &S, int plan, int parity, int64_t k0, int n,
                             cudaStream_t st) {
   switch (plan) {
+    case kResidentOne:
     case kResidentSmall:
     case kResidentCluster: return launch_resident_c<Small, true>(P, S, plan == kResidentCluster, parity, k0, n, st);
     case kResidentLarge: return launch_resident_c<Large, false>(P, S, false, parity, k0, n, st);
