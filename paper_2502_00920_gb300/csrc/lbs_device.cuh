@@ -777,7 +777,7 @@ struct TileCfg : TileGeom<TX_, TY_, NTY_> {
 // first moments sum_q e_q g_q (own node, post-collision at k) and
 // sum_q e_q f_q (streamed, at k + 1).  EDGE: wrap, walls and boundary rules;
 // LIN: the two-point wall extrapolation (lattices with P.extrap set).
-template <class Pr, bool EDGE, bool LIN, bool COH = false>
+template <class Pr, bool EDGE, bool LIN>
 __device__ __forceinline__ void gather(const Params &P, const typename Pr::gs *g, const typename Pr::real *bnd,
                                        const EdgeType<typename Pr::real, LIN> (*sev)[2], int x, int y,
                                        const Coef<typename Pr::real> &k, typename Pr::real f[9],
@@ -792,9 +792,9 @@ __device__ __forceinline__ void gather(const Params &P, const typename Pr::gs *g
   // the frame tiles, which lie within three nodes of a wall or of the end)
   if (!EDGE || (x >= 1 && x <= P.nx - 2 && y >= 1 && y <= P.ny - 2)) {
 #pragma unroll
-    for (int q = 0; q < 9; ++q) f[q] = gld<COH>(g, q * plane + idx - ex(q) - (ptrdiff_t)ey(q) * P.pitch, inv);
+    for (int q = 0; q < 9; ++q) f[q] = gload(g, q * plane + idx - ex(q) - (ptrdiff_t)ey(q) * P.pitch, inv);
 #pragma unroll
-    for (int q = 1; q < 9; ++q) g0[q] = gld<COH>(g, q * plane + idx, inv);
+    for (int q = 1; q < 9; ++q) g0[q] = gload(g, q * plane + idx, inv);
     g0[0] = 0;
   } else {
     // all loads without branches in between, so that they are in flight
@@ -804,17 +804,17 @@ __device__ __forceinline__ void gather(const Params &P, const typename Pr::gs *g
     stream_sides(y, P.ny, P.per_y, yb, yf);
     walls_of(P, x, y, xw, yw);
     R wn[4];
-    wall_n<COH>(P, bnd, xw, yw, x, y, wn);
+    wall_n<false>(P, bnd, xw, yw, x, y, wn);
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
       const int sx = ex(q) > 0 ? xb : (ex(q) < 0 ? xf : x), sy = ey(q) > 0 ? yb : (ey(q) < 0 ? yf : y);
-      g0[q] = gld<COH>(g, q * plane + idx, inv);
-      f[q] = gld<COH>(g, q * plane + (size_t)sy * P.pitch + sx, inv);
+      g0[q] = gload(g, q * plane + idx, inv);
+      f[q] = gload(g, q * plane + (size_t)sy * P.pitch + sx, inv);
     }
     if (xw >= 0 || yw >= 0) {
       if constexpr (LIN)
-        wall_rules<R, typename Pr::gs, COH>(P, bnd, g, sev, x, y, xw, yw, wn, g0, crosses_x(xw) | crosses_y(yw),
-                                                 f, k.ics2, k.cj);
+        wall_rules<R, typename Pr::gs, false>(P, bnd, g, sev, x, y, xw, yw, wn, g0, crosses_x(xw) | crosses_y(yw),
+                                             f, k.ics2, k.cj);
       else
         wall_rules_own<R>(P, xw, yw, sev, k.ics2, k.cj, wn, g0, f);
     }
