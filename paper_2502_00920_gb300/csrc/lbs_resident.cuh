@@ -8,19 +8,12 @@
 
 namespace lbs {
 
-// A tile of TX x TY nodes whose block has a thread for every node of the tile
-// plus its 2-node halo (R2): entry e < OWN is own node e, the rest are the ring.
 template <class Pr, int TX_, int TY_>
-struct ResCfg {
+struct ResCfg : ResGeom<TX_, TY_> {
   using PrT = Pr;
   using real = typename Pr::real;
   using us = typename Pr::us;
   using gs = typename Pr::gs;
-  static constexpr int TX = TX_, TY = TY_;
-  static constexpr int R2W = TX + 4, R2H = TY + 4, R1W = TX + 2, R1H = TY + 2;
-  static constexpr int OWN = TX * TY, NRING = R2W * R2H - OWN;
-  static constexpr int NT = (R2W * R2H + 31) / 32 * 32;
-  static_assert(NT <= 1024, "one thread per node of R2");
 };
 
 // Barrier over the blocks of one cooperative launch: every block adds one to
@@ -95,12 +88,7 @@ __global__ void __launch_bounds__(C::NT) resident_kernel(const Params P, const C
   bool in = false, own = false;
   us uu;
   if (e < C::OWN + C::NRING) {
-    if (e < C::OWN) {
-      rx = e % C::TX + 2;
-      ry = e / C::TX + 2;
-    } else {
-      ring_pos<C>(e - C::OWN, rx, ry);
-    }
+    resident_pos<C>(e, rx, ry);
     x = x0 - 2 + rx;
     y = y0 - 2 + ry;
     own = e < C::OWN && x < P.nx && y < P.ny;

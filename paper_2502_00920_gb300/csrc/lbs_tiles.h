@@ -1,10 +1,11 @@
 // Index arithmetic of the tiled kernels: the D2Q9 directions, which node a
 // thread updates, where its streaming sources and finite-difference taps lie,
 // which shared-memory and boundary side-array entries it touches, how the
-// frame tiles are enumerated and where the TMA boxes start.  Plain C++ with
-// no device code: the kernels call these functions, and a host program
-// (tests/c/tile_bounds.cc) drives them over every tile shape and over ragged
-// and degenerate lattices to check each index against its allocation.
+// frame tiles are enumerated, where the TMA boxes start and what the warp
+// columns cover.  Plain C++ with no device code: the kernels call these
+// functions, and host programs (tests/c/tile_bounds.cc, resident_bounds.cc,
+// column_bounds.cc) drive them over every tile shape and over ragged and
+// degenerate lattices to check each index against its allocation.
 //
 // The lattice type G of the templates is anything with the members
 //   nx, ny (nodes), pitch (row pitch in elements), per_x, per_y (periodic
@@ -66,6 +67,27 @@ LBS_HD void ring_pos(int r, int &rx, int &ry) {
   }
 }
 
+// A resident tile of TX x TY nodes: its block has a thread for every node of the
+// tile plus its 2-node halo (R2); entry e < OWN is own node e, the rest are the
+// ring.  N on R1 and the own nodes go to the first threads.
+template <int TX_, int TY_>
+struct ResGeom {
+  static constexpr int TX = TX_, TY = TY_;
+  static constexpr int R2W = TX + 4, R2H = TY + 4, R1W = TX + 2, R1H = TY + 2;
+  static constexpr int OWN = TX * TY, NRING = R2W * R2H - OWN;
+  static constexpr int NT = (R2W * R2H + 31) / 32 * 32;
+  static_assert(NT <= 1024, "one thread per node of R2");
+};
+template <class C>
+LBS_HD void resident_pos(int e, int &rx, int &ry) {
+  if (e < C::OWN) {
+    rx = e % C::TX + 2;
+    ry = e / C::TX + 2;
+  } else {
+    ring_pos<C>(e - C::OWN, rx, ry);
+  }
+}
+
 // wrap (periodic axis) or reject a node coordinate; false outside a wall.
 // Coordinates handed in lie within one lattice length of the lattice.
 template <class G>
@@ -83,7 +105,9 @@ LBS_HD bool locate(const G &P, int &x, int &y) {
 
 // Source (sx, sy) of population q streaming into node (x, y) of the lattice:
 // (x - ex(q), y - ey(q)), wrapped on a periodic axis.  False where the source
-// lies beyond a wall (the boundary rules then supply f_q).
+// lies beyond a wall (the boundary rules then supply f_q).  The definition that
+// tile_bounds.cc holds the tiles against; the kernels take the same sources
+// from stream_sides and the crosses_x / crosses_y masks, all q at once.
 template <class G>
 LBS_HD bool stream_source(const G &P, int x, int y, int q, int &sx, int &sy) {
   sx = x - ex(q);
