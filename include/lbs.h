@@ -316,7 +316,9 @@ size_t lbs_footprint(const lbs_lattice *lat);
 
 /* First Piola-Kirchhoff stress P(H) and the constitutive source tensor
  * N(H) = P(H) + Pi(H), Pi(H) = -mu (H + H^T + tr H I) (Eq. source), evaluated
- * on the host with the same formulas the kernels use (double precision).
+ * on the host with the kernels' formulas (double precision; the double-
+ * precision kernels take neo-Hooke from the displacement differences, which
+ * agrees to rounding).
  * H, P, N: row-major 2x2. */
 int lbs_constitutive(int32_t model, double lam, double mu, const double H[4], double P[4], double N[4]);
 

@@ -243,7 +243,7 @@ __host__ __device__ inline bool constitutive_n(int model, R lam, R mu, const R H
 // N in the compute type; the FP32 kernels evaluate neo-Hooke in double where
 // J < 1/2 (near det F -> 0 the 1/J terms lose float accuracy)
 template <class R>
-__device__ __forceinline__ void material(const Params &P, R lam, R mu, const R H[4], R N[4]) {
+__host__ __device__ __forceinline__ void material(const Params &P, R lam, R mu, const R H[4], R N[4]) {
   if constexpr (sizeof(R) == 4) {
     if (!constitutive_n<R>(P.model, lam, mu, H, N, R(0.5))) {
       double Hd[4] = {H[0], H[1], H[2], H[3]}, Nd[4];
@@ -301,7 +301,7 @@ struct Pick<false, X, Y> {
 template <class R, bool LIN>
 using EdgeType = typename Pick<LIN, double, R>::type;
 constexpr int kEdgeEntries = 8;
-__device__ __forceinline__ int edge_corner(int xw, int yw) { return 4 + (xw == kRight ? 1 : 0) + (yw == kTop ? 2 : 0); }
+__host__ __device__ __forceinline__ int edge_corner(int xw, int yw) { return 4 + (xw == kRight ? 1 : 0) + (yw == kTop ? 2 : 0); }
 
 template <class T>
 __device__ inline void edge_entry(const Params &P, int i, int64_t k, T out[2]) {
@@ -502,7 +502,7 @@ __device__ void wall_rules(const Params &P, const R *bnd, const G *g, const doub
 // zero.  (The general form above converts the values from double per node and
 // multiplies by the zeros; in FP64 those products are pipe slots.)
 template <class R>
-__device__ __forceinline__ void wall_rules_own(const Params &P, int xw, int yw, const R (*sev)[2], R ics2, R cj,
+__host__ __device__ __forceinline__ void wall_rules_own(const Params &P, int xw, int yw, const R (*sev)[2], R ics2, R cj,
                                                const R wn[4], const R g0[9], R f[9]) {
   const unsigned crossx = crosses_x(xw), crossy = crosses_y(yw), mask = crossx | crossy;
   const bool dirx = xw >= 0 && P.etype[xw] == LBS_DIRICHLET, diry = yw >= 0 && P.etype[yw] == LBS_DIRICHLET;
@@ -625,7 +625,7 @@ __host__ __device__ __forceinline__ CollideK<R> collide_k(R omega, R sigma, R sc
 // (-omega o57 = omega (tx + ty) / 12): 39 slots a node where forming t57, t68
 // and their forcing apart took 47.
 template <class R>
-__device__ __forceinline__ void collide(R f[9], R Sx, R Sy, const CollideK<R> &K) {
+__host__ __device__ __forceinline__ void collide(R f[9], R Sx, R Sy, const CollideK<R> &K) {
   const R s13 = f[1] + f[3], s24 = f[2] + f[4], s57 = f[5] + f[7], s68 = f[6] + f[8];
   const R d13 = f[1] - f[3], d24 = f[2] - f[4], d57 = f[5] - f[7], d68 = f[6] - f[8];
   // (the products by 2 and 4 are exact)
@@ -722,7 +722,7 @@ __host__ __device__ inline Coef<R> make_coef(const Params &P) {
 // one-sided difference is doubled first, exactly); otherwise H is formed and
 // handed to material().
 template <class R>
-__device__ __forceinline__ void stress_n(const Params &P, const Coef<R> &c, R dxx, R dxy, R dyx, R dyy, bool onex,
+__host__ __device__ __forceinline__ void stress_n(const Params &P, const Coef<R> &c, R dxx, R dxy, R dyx, R dyy, bool onex,
                                          bool oney, R N[4]) {
   if constexpr (sizeof(R) == 8) {
     if (P.model == LBS_NH) {
