@@ -25,6 +25,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
+#include <string.h>
 
 #include "lbs_internal.h"
 
@@ -686,7 +687,7 @@ struct Coef {
   R sbx, sby;    // rho0 b
   // the same as the collision takes the source: times sigma/9 in FP64
   R idxs, hdxs, sbxs, sbys;
-  R h2, c1;      // hdx^2, lam / (2 mu) (FP64 neo-Hooke)
+  R h2, c1;      // hdx^2 (0: out of range), lam / (2 mu) (FP64 neo-Hooke)
   R ics2, cj;    // 1 / cs^2 and c / cs^2 in storage units of g (wall rules)
   CollideK<R> K;
 };
@@ -710,9 +711,17 @@ __host__ __device__ inline Coef<R> make_coef(const Params &P) {
   k.hdxs = R(0.5) * k.idxs;
   k.sbxs = k.sbx * src;
   k.sbys = k.sby * src;
-  k.h2 = k.hdx * k.hdx;
+  // (the products of differences and hdx^2 stay in range; else H is formed first)
+  k.h2 = (double)k.hdx > 1e-140 && (double)k.hdx < 1e140 ? k.hdx * k.hdx : R(0);
   k.c1 = R(0.5) * k.lam / k.mu;
   return k;
+}
+
+// whether a coefficient is not +0, without a slot of the FP64 pipe
+__host__ __device__ __forceinline__ bool set_bits(double v) {
+  int64_t b;
+  memcpy(&b, &v, sizeof(b));
+  return b != 0;
 }
 
 // N of a node from the differences of u over two spacings (dxx = the
@@ -725,7 +734,7 @@ template <class R>
 __host__ __device__ __forceinline__ void stress_n(const Params &P, const Coef<R> &c, R dxx, R dxy, R dyx, R dyy, bool onex,
                                          bool oney, R N[4]) {
   if constexpr (sizeof(R) == 8) {
-    if (P.model == LBS_NH) {
+    if (P.model == LBS_NH && set_bits(c.h2)) {
       if (onex) {
         dxx += dxx;
         dxy += dxy;

@@ -146,3 +146,17 @@ def test_wall_rules(forms, real):
     assert got.shape == (len(cases), 9)
     assert (np.abs(got - np.array(want)) <= np.array(bound)).all()
     assert (np.array(bound) > 0).any(axis=1).all()
+
+
+@pytest.mark.parametrize("dx", [2.0 ** -530, 1e-150, 1e-100, 1e100, 1e150, 2.0 ** 530])
+def test_neo_hooke_at_any_spacing(forms, oracle_mod, dx):
+    """The double-precision form squares 1 / (2 dx) where that stays in range."""
+    rng = np.random.default_rng(4)
+    mu, lam = 0.4, 0.3
+    H = rng.normal(0.0, 0.05, (20, 4))
+    got = forms("double", "stress", [[1, lam, mu, dx, *(np.array([h[0], h[2], h[1], h[3]]) * 2 * dx), 0, 0] for h in H])
+    for h, n in zip(H, got):
+        want = oracle_mod.first_piola("nh", lam, mu, h).reshape(4) + oracle_mod.pi_of_h(mu, h).reshape(4)
+        m = 2 * np.abs(h).max()
+        J = (1 + h[0]) * (1 + h[3]) - h[1] * h[2]
+        assert np.abs(n - want).max() <= 64 * EPS["double"] * (lam + 2 * mu) * m * (1 + m) ** 2 / J + 1e-14 * (1 + lam + mu)
