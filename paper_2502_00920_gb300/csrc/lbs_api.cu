@@ -1025,6 +1025,8 @@ int lbs_load(lbs_handle *h, const void *buf, size_t bytes) {
   if (bytes < sizeof(CkptHeader) + sz.g + sz.u + sz.b || hd.k < 0) return fail(LBS_EINVAL, "checkpoint truncated");
   LBS_CK(cudaStreamSynchronize(h->stream));
   const char *in = (const char *)buf + sizeof(CkptHeader);
+  // (the server's batches take the state of iteration k from buffers [k & 1])
+  h->parity = (int)(hd.k & 1);
   LBS_CK(cudaMemcpy(h->g[h->parity], in, sz.g, cudaMemcpyHostToDevice));
   LBS_CK(cudaMemcpy(h->u[h->parity], in + sz.g, sz.u, cudaMemcpyHostToDevice));
   LBS_CK(cudaMemcpy(h->b[h->parity], in + sz.g + sz.u, sz.b, cudaMemcpyHostToDevice));
