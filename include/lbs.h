@@ -286,11 +286,11 @@ int lbs_selftest_bounded_wait(uint32_t tx_bytes, uint32_t polls, int32_t *timed_
 
 /* The same for the barrier between the blocks of a resident launch (lbs_step):
  * launches the handle's next two iterations with one arrival taken from the
- * barrier's count, so that every block gives up after `polls` polls and
- * returns.  Asynchronous: the handle reports LBS_ETIMEOUT (lbs_sync) and takes
- * a new state like any other.  Errors: LBS_EINVAL (polls == 0, or a lattice
- * whose launches have no such barrier), LBS_ECUDA. */
-int lbs_selftest_resident_wait(lbs_handle *h, uint32_t polls);
+ * barrier's count, so that every block gives up after its number of polls (under
+ * a second) and returns.  Asynchronous: the handle reports LBS_ETIMEOUT
+ * (lbs_sync) and takes a new state like any other.  Errors: LBS_EINVAL (NULL, or
+ * a lattice whose launches have no such barrier), LBS_ECUDA. */
+int lbs_selftest_resident_wait(lbs_handle *h);
 
 /* The handle's current tile variant (LBS_EINVAL for a null handle). */
 int32_t lbs_variant(const lbs_handle *h);

@@ -307,7 +307,7 @@ StepPtrs ptrs(const lbs_handle *h, int parity, const int64_t *kptr, int64_t koff
 }
 
 // (mon_out[7] holds the barrier's counters)
-ResidentPtrs resident_ptrs(const lbs_handle *h, uint32_t polls) {
+ResidentPtrs resident_ptrs(const lbs_handle *h) {
   ResidentPtrs s;
   for (int i = 0; i < 2; ++i) {
     s.g[i] = h->g[i];
@@ -316,7 +316,6 @@ ResidentPtrs resident_ptrs(const lbs_handle *h, uint32_t polls) {
   }
   s.bar = (unsigned *)(h->mon_out + 7);
   s.err = h->errdev;
-  s.polls = polls;
   return s;
 }
 
@@ -704,7 +703,7 @@ int lbs_step(lbs_handle *h, int64_t n) {
         } while (run < n && run < kResidentMost && !(h->mon_interval > 0 && h->k + run >= h->next_mon));
       }
       const int m = (int)std::min<int64_t>(run, kResidentMost);
-      const cudaError_t e = h->L->resident(h->P, resident_ptrs(h, kMaxBarrierPolls), h->resident, h->parity, h->k, m, h->stream);
+      const cudaError_t e = h->L->resident(h->P, resident_ptrs(h), h->resident, h->parity, h->k, m, h->stream);
       if (e != cudaSuccess && h->resident == kResidentCluster) {
         // the cluster is refused: the grid barrier instead (which reports what
         // else may be wrong)
@@ -797,14 +796,14 @@ int lbs_sync(lbs_handle *h) {
   return rc ? rc : check_monitor(h, true);
 }
 
-int lbs_selftest_resident_wait(lbs_handle *h, uint32_t polls) {
-  if (!h || polls == 0) return fail(LBS_EINVAL, "bad self-test arguments");
+int lbs_selftest_resident_wait(lbs_handle *h) {
+  if (!h) return fail(LBS_EINVAL, "null handle");
   if (h->resident != kResidentSmall && h->resident != kResidentLarge)
     return fail(LBS_EINVAL, "no grid barrier in this lattice's launches");
   // one arrival too few: the count starts at -1, and two iterations of a grid
   // of at least two blocks wait for all of them once
   LBS_CK(cudaMemsetAsync(h->mon_out + 7, 0xff, sizeof(unsigned), h->stream));
-  LBS_CK(h->L->resident(h->P, resident_ptrs(h, polls), h->resident, h->parity, h->k, 2, h->stream));
+  LBS_CK(h->L->resident(h->P, resident_ptrs(h), h->resident, h->parity, h->k, 2, h->stream));
   h->launches += 1;
   h->k += 2;
   return LBS_OK;

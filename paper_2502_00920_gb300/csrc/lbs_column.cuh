@@ -80,7 +80,9 @@ static __device__ __noinline__ float4 nh_wide(double lam, double mu, float h11, 
 }
 
 // constitutive_n<float> on two nodes: the same operations, with negations
-// folded into factors (exact)
+// folded into factors (exact).  This and collide_v2 follow the functions they
+// restate operation by operation (tests/test_column_gpu.py compares the bits):
+// a change of either belongs in both.
 __device__ __forceinline__ void stress_v2(const Params &P, const Coef<float> &c, Two dxx, Two dxy, Two dyx, Two dyy,
                                           Two N[4]) {
   const Two h = two(c.hdx);

@@ -67,9 +67,6 @@ struct StepPtrs {
 // behind a grid barrier.
 enum { kResidentNone = 0, kResidentOne, kResidentSmall, kResidentCluster, kResidentLarge };
 
-// polls of a resident launch's barrier at most (seconds)
-constexpr uint32_t kMaxBarrierPolls = 1u << 22;
-
 // Device pointers of one lattice for a resident launch: both buffers of each
 // state array, the barrier's two counters (zero between launches) and the
 // error flag.
@@ -77,7 +74,6 @@ struct ResidentPtrs {
   void *g[2], *u[2], *b[2];
   unsigned *bar;
   int *err;
-  uint32_t polls;  // of the barrier, after which a block gives up
 };
 
 struct TileShape {

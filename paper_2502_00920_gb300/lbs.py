@@ -100,7 +100,7 @@ SIGNATURES = {
     "lbs_variant": (ctypes.c_int32, [_vp]),
     "lbs_selftest_bounded_wait": (ctypes.c_int, [ctypes.c_uint32, ctypes.c_uint32, _i32p,
                                                  ctypes.POINTER(ctypes.c_double)]),
-    "lbs_selftest_resident_wait": (ctypes.c_int, [_vp, ctypes.c_uint32]),
+    "lbs_selftest_resident_wait": (ctypes.c_int, [_vp]),
     "lbs_checkpoint_bytes": (ctypes.c_size_t, [_vp]),
     "lbs_save": (ctypes.c_int, [_vp, ctypes.c_void_p, ctypes.c_size_t]),
     "lbs_load": (ctypes.c_int, [_vp, ctypes.c_void_p, ctypes.c_size_t]),
@@ -353,10 +353,10 @@ class Simulation:
     def variant(self) -> int:
         return int(lib().lbs_variant(self._h))
 
-    def selftest_resident_wait(self, polls: int):
+    def selftest_resident_wait(self):
         """A resident launch whose barrier runs out (see
         lbs_selftest_resident_wait)."""
-        check(lib().lbs_selftest_resident_wait(self._h, int(polls)))
+        check(lib().lbs_selftest_resident_wait(self._h))
 
     # -- checkpoint / resume
     def save(self) -> np.ndarray:
