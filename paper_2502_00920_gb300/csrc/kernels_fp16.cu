@@ -119,8 +119,8 @@ void coef(const Params &p, void *out) {
 
 // resident launches: the tiles and lines of single precision (us per iteration
 // on walled neo-Hooke lattices, one lattice alone / three side by side, against
-// launching every iteration from a graph: 40 x 40 10.1 / 3.5 -> 2.8 / 0.94,
-// 128 x 128 10.5 / 3.7 -> 2.8 / 1.6, 256 x 256 10.8 / 4.8 -> 3.7 / 3.6)
+// launching every iteration from a graph: 40 x 40 11.4 / 3.9 -> 2.7 / 0.90,
+// 128 x 128 11.4 / 4.0 -> 3.0 / 2.1, 256 x 256 11.8 / 5.1 -> 3.7 / 3.8)
 using RS = ResCfg<P, 16, 8>;
 using RL = ResCfg<P, 32, 14>;
 int resident_large(const Params &p) { return p.extrap ? resident_sms() / 2 : resident_sms(); }

@@ -140,13 +140,13 @@ void coef(const Params &p, void *out) {
 
 // resident launches (us per iteration on walled neo-Hooke lattices, one lattice
 // alone / three advancing side by side; launching every iteration from a graph
-// before them): 32 x 32 9.1 / 3.1 -> 2.9 / 0.95 and 128 x 128 9.5 / 3.3 ->
-// 2.9 / 1.6 on 16 x 8 tiles, 160 x 160 10.7 / 4.2 -> 4.0 / 1.4 and 256 x 256
-// 9.5 / 4.2 -> 3.6 / 3.5 on 32 x 14 tiles (21 warps at 80 registers, one block
+// before them): 32 x 32 10.7 / 3.7 -> 2.2 / 0.75 and 128 x 128 10.4 / 3.6 ->
+// 2.6 / 1.9 on 16 x 8 tiles, 160 x 160 10.5 / 3.8 -> 3.6 / 2.4 and 256 x 256
+// 10.5 / 4.5 -> 3.6 / 3.6 on 32 x 14 tiles (21 warps at 80 registers, one block
 // per SM; 32 x 16 tiles, 23 warps, 3.7 / 3.65: they would reach 78 000 nodes
 // instead of 68 000, and no size in between was measured; two nodes a thread, to
 // fit two blocks, spilled: 6.4 / 4.0).
-// Two-point wall extrapolation: 160 x 40 11.8 / 4.5 -> 4.7 / 1.6; its large
+// Two-point wall extrapolation: 160 x 40 11.8 / 4.1 -> 4.5 / 1.6; its large
 // tiles lose beside others once they fill the GPU (391 x 173 12.3 / 5.4 -> 7.2
 // / 7.1), so they stop at half.
 using RS = ResCfg<P, 16, 8>;

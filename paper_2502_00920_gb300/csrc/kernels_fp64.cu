@@ -72,8 +72,8 @@ void coef(const Params &p, void *out) {
 
 // resident launches (us per iteration on walled neo-Hooke lattices, one lattice
 // alone / three side by side, against launching every iteration from a graph):
-// 40 x 40 26.4 / 8.9 -> 8.3 / 2.7, 160 x 40 26.2 / 8.8 -> 7.5 / 3.5 and 96 x 96
-// 31.6 / 11.1 -> 9.1 / 6.6 on 8 x 8 tiles, 128 x 128 31.6 / 11.4 -> 19.7 / 9.9 on
+// 40 x 40 27.5 / 9.2 -> 7.5 / 2.5, 160 x 40 26.2 / 8.8 -> 7.5 / 3.5 and 96 x 96
+// 30.1 / 10.2 -> 7.5 / 6.7 on 8 x 8 tiles, 128 x 128 30.3 / 10.3 -> 15.4 / 10.2 on
 // 16 x 16 tiles.  FP64 operations bound both (a warp's operation holds its
 // scheduler's FP64 unit for tens of cycles), so a tile's halo is dear: past
 // half the SMs the 16 x 16 tiles lose beside others (160 x 160 31.6 / 15.1 ->

@@ -12,7 +12,7 @@
 // work. 16384^2 periodic, ms per iteration: FP32 4.20 -> 3.27 (two iterations
 // per launch), FP16 storage 3.38 -> 3.00. What bounds it now: instruction
 // issue and latency with the 12 warps an SM holds at 168 registers (4096^2
-// FP32: issue 57 %, shared-memory pipe 67 %, DRAM 4.1 TB/s). Packed FP32
+// FP32: issue 59 %, shared-memory pipe 63 %, DRAM 4.1 TB/s). Packed FP32
 // instructions (add.f32x2 and so on) measured the same (two issue cycles each)
 // and ptxas fuses their products into sums, which changes the rounding.
 #pragma once

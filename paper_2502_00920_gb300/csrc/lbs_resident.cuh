@@ -58,13 +58,14 @@ constexpr int kSevBatch = 32;
 // them.  Where a block gives up waiting, the counters stay as they are and the
 // error flag is set; a launch that finds it set does nothing, until setting the
 // state anew clears both.
-// What bounds an iteration: latency. Of the 2.9 us on a 16 x 8 FP32 tile the
-// grid barrier takes 1.0, the loads from L2 0.4, the three phases the rest (FP64:
-// its operations' own latency, some 300 cycles each in chains of about 35).
+// What bounds an iteration: latency. Of the 2.6 us of 128 x 128 FP32 (128 blocks)
+// the grid barrier alone takes 1.1, and the schedulers issue 12 % of the cycles;
+// in FP64 a dependent operation takes 303 cycles, some 40 of them in a row in
+// the 7.5 us of 40 x 40.
 // CLUSTER: the grid is one thread-block cluster, whose hardware barrier takes
-// 0.5 us where the grid barrier takes 1.0 (it orders global memory within the
-// cluster, and cannot run out: a cluster's blocks run together). 32 x 32 FP32:
-// 0.34 -> 0.30 ms for 400 iterations among three lattices.
+// 0.5 us where the grid barrier takes 0.9 at 16 blocks (it orders global memory
+// within the cluster, and cannot run out: a cluster's blocks run together).
+// 32 x 32 FP32: 0.34 -> 0.30 ms for 400 iterations among three lattices.
 template <class C, bool LIN, bool CLUSTER>
 __global__ void __launch_bounds__(C::NT) resident_kernel(const Params P, const Coef<typename C::real> c,
                                                          const ResidentPtrs S, int parity, int64_t k0, int n,
