@@ -262,11 +262,11 @@ __global__ void reset_state_kernel(int64_t *k, double *mon_out, int *err) {
 }
 
 cudaError_t queue_flag(lbs_handle *h) {
-  return cudaMemcpyAsync(h->mon_host + 7, h->errdev, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+  return cudaMemcpyAsync(h->mon_host + kMonFlag, h->errdev, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
 }
 int check_flag(lbs_handle *h) {
   int gave_up;
-  memcpy(&gave_up, h->mon_host + 7, sizeof(int));
+  memcpy(&gave_up, h->mon_host + kMonFlag, sizeof(int));
   if (gave_up) h->gave_up = true;
   if (!h->gave_up) return LBS_OK;
   set_error("a kernel gave up waiting for its tile copies or its other blocks: the state is not advanced "
@@ -385,8 +385,8 @@ int check_monitor(lbs_handle *h, bool wait) {
 int launch_monitor_async(lbs_handle *h) {
   LBS_CK(h->L->monitor(h->P, h->g[h->parity], h->u[h->parity], h->mon_partials, monitor_blocks(h->P), h->mon_out,
                        h->k, h->stream));
-  LBS_CK(cudaMemcpyAsync(h->mon_host, h->mon_out, 7 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-  LBS_CK(queue_flag(h));
+  // (with the flag, which lies behind)
+  LBS_CK(cudaMemcpyAsync(h->mon_host, h->mon_out, (kMonFlag + 1) * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
   LBS_CK(cudaEventRecord(h->mon_event, h->stream));
   h->launches += 2;
   h->mon_pending = true;
@@ -566,7 +566,7 @@ int lbs_create(const lbs_lattice *lat, const lbs_material *mat, const lbs_bcs *b
       ok = h->mon_block != nullptr;
     }
   }
-  if (ok && cudaMallocHost(&h->mon_host, 8 * sizeof(double)) != cudaSuccess) {
+  if (ok && cudaMallocHost(&h->mon_host, (kMonFlag + 1) * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();
     h->mon_host = nullptr;
     ok = false;
@@ -590,7 +590,7 @@ int lbs_create(const lbs_lattice *lat, const lbs_material *mat, const lbs_bcs *b
   h->mon_out = (double *)(mb + (size_t)monitor_blocks(h->P) * 5 * sizeof(double));
   h->kdev = (int64_t *)(h->mon_out + 8);
   h->zero_dev = h->kdev + 1;
-  h->errdev = (int *)(h->kdev + 2);
+  h->errdev = (int *)(h->mon_out + kMonFlag);  // (kdev + 2)
   h->sev = h->kdev + 3;
   h->bytes = lay.total;
   rc = select_variant(h, h->L->default_variant(h->P));

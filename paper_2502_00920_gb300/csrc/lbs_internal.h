@@ -76,6 +76,9 @@ struct ResidentPtrs {
   int *err;
 };
 
+// place of the error flag behind a handle's monitor values, in doubles
+constexpr int kMonFlag = 10;
+
 struct TileShape {
   int tx, ty;
 };
@@ -199,7 +202,7 @@ struct lbs_handle {
   double *mon_out;          // device: bad, max|u|, mx, my, mass, flag
   int64_t *kdev;            // device iteration base used by graph replays
   int64_t *zero_dev;        // device constant 0 (direct launches)
-  double *mon_host;         // pinned copy of mon_out's first seven, then of the flag
+  double *mon_host;         // pinned copy of mon_out and, at kMonFlag, of the error flag
   cudaEvent_t mon_event;
   bool mon_pending;
   int64_t mon_k;            // iteration of the pending monitor
@@ -216,7 +219,7 @@ struct lbs_handle {
   int cfl_warn;
   int64_t launches;         // kernels launched for this handle
   void *sev;                // edge table of kEdgeBatch iterations
-  int *errdev;              // device flag: a bounded wait in a kernel gave up
+  int *errdev;              // device flag: a bounded wait in a kernel gave up (mon_out + kMonFlag)
   bool gave_up;             // the flag was seen set (until the state is set anew)
   CUtensorMap tm_g[2];      // TMA descriptors of g[0], g[1] and u[0], u[1]
   CUtensorMap tm_u[2];      //   for the current variant (TMA variants only)
